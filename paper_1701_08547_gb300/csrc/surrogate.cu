@@ -20,6 +20,7 @@
 #include "tc_gemm.cuh"
 #include "tc_mlp.cuh"
 #include "tc_mlp_bwd.cuh"
+#include "tc_mlp_train.cuh"
 #include "tc_wgrad.cuh"
 #include "tune_internal.h"
 
@@ -522,20 +523,15 @@ int refresh_fp8(tune_surrogate* h, cudaStream_t s)
     return TUNE_OK;
 }
 
-template <bool FP8, bool TRAIN = false>
-int launch_fused(const CUtensorMap& tx, const CUtensorMap& tw1, const CUtensorMap& tw, const CUtensorMap& th,
-                 const tcm::Args& g, unsigned grid, cudaStream_t s)
+template <bool FP8>
+int launch_fused(const CUtensorMap& tx, const CUtensorMap& tw1, const CUtensorMap& tw, const tcm::Args& g, unsigned grid,
+                 cudaStream_t s)
 {
     constexpr int smem = tcm::Cfg<FP8>::smem;
     static std::atomic<uint64_t> attr{0};
-    const int rc = smem_attr(tcm::mlp_infer_kernel<FP8, TRAIN>, smem, attr, "surrogate: fused smem attribute");
+    const int rc = smem_attr(tcm::mlp_infer_kernel<FP8>, smem, attr, "surrogate: fused smem attribute");
     if (rc) return rc;
-    if constexpr (TRAIN)  // a step of the training chain (pdl.cuh)
-        TUNE_CUDA_TRY(pdl::launch_dep(tcm::mlp_infer_kernel<FP8, TRAIN>, dim3(grid), dim3(tcm::kThreads), smem, s, tx,
-                                      tw1, tw, th, g),
-                      "surrogate: fused launch");
-    else
-        tcm::mlp_infer_kernel<FP8, TRAIN><<<grid, tcm::kThreads, smem, s>>>(tx, tw1, tw, th, g);
+    tcm::mlp_infer_kernel<FP8><<<grid, tcm::kInferThreads, smem, s>>>(tx, tw1, tw, g);
     TUNE_CUDA_TRY(cudaGetLastError(), "surrogate: fused launch");
     return TUNE_OK;
 }
@@ -586,16 +582,10 @@ int fused_forward(tune_surrogate* h, const __nv_bfloat16* feats, int64_t n, floa
     g.wscale_half = h->wscale_half;
     g.pred = pred;
     g.pred_stride = n;
-    for (int l = 0; l < NL; ++l) {
-        g.g_out[l] = nullptr;
-        g.h_out[l] = nullptr;
-    }
-    g.act_stride = 0;
     g.status = h->status;
     const long long sms = tune::device_sm_count();
     const unsigned grid = (unsigned)(g.units < sms ? g.units : sms);
-    // (the activation map is used by the training variant only)
-    return fp8 ? launch_fused<true>(tx, tw1, tw, tx, g, grid, s) : launch_fused<false>(tx, tw1, tw, tx, g, grid, s);
+    return fp8 ? launch_fused<true>(tx, tw1, tw, g, grid, s) : launch_fused<false>(tx, tw1, tw, g, grid, s);
 }
 
 // Training forward of rows [0, n_pad) of the current batch (h->xb) through the fused kernel
@@ -629,7 +619,8 @@ int fused_train_forward(tune_surrogate* h, int n_pad, cudaStream_t s)
     const cuuint32_t hb[4] = {16, tcm::kRows, 1, 1};
     rc = make_map_nd(&th, u64, 4, h->H[0], hd, hs, hb);
     if (rc) return rc;
-    tcm::Args g;
+    tcm::TrainArgs a;
+    tcm::Args& g = a.f;
     g.n = n_pad;
     g.members = h->members;
     g.units = (long long)(n_pad / tcm::kRows) * h->members;
@@ -641,15 +632,19 @@ int fused_train_forward(tune_surrogate* h, int n_pad, cudaStream_t s)
     g.wscale_half = h->wscale_half;
     g.pred = h->y;
     g.pred_stride = h->batch;
-    for (int l = 0; l < NL; ++l) {
-        g.g_out[l] = h->G[l];
-        g.h_out[l] = h->H[l];
-    }
-    g.act_stride = (long long)h->batch * WID;
     g.status = h->status;
+    for (int l = 0; l < NL; ++l) a.g_out[l] = h->G[l];
+    a.h4_out = h->H[NL - 1];
+    a.act_stride = (long long)h->batch * WID;
+    constexpr int smem = tcm::Cfg<false>::smem;
+    static std::atomic<uint64_t> attr{0};
+    rc = smem_attr(tcm::mlp_train_kernel, smem, attr, "surrogate: training forward smem attribute");
+    if (rc) return rc;
     const long long sms = tune::device_sm_count();
     const unsigned grid = (unsigned)(g.units < sms ? g.units : sms);
-    return launch_fused<false, true>(tx, tw1, tw, th, g, grid, s);
+    TUNE_CUDA_TRY(pdl::launch_dep(tcm::mlp_train_kernel, dim3(grid), dim3(tcm::kThreads), smem, s, tx, tw1, tw, th, a),
+                  "surrogate: training forward launch");
+    return TUNE_OK;
 }
 
 // Input gradients of layers 4, 3 and 2 in one persistent launch (tc_mlp_bwd.cuh):
