@@ -33,7 +33,7 @@
 #include <limits>
 #include <mutex>
 
-#include "eval_common.cuh"
+#include "eval_tables.cuh"
 #include "pdl.cuh"
 #include "tune_internal.h"
 
@@ -43,33 +43,9 @@ using namespace tune_dev;
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
-constexpr int kMaxB = 32;  // blocks per SM supported by the tables
-constexpr int kIparStride = 17;  // words per ipar row (16 grid positions and one of padding)
 constexpr unsigned kFull = 0xffffffffu;
 
-
-
 constexpr int kMaxArch = 8;  // architecture rows of one tune_eval_archs call
-
-struct CtaTables {
-    // (waves*slots)/(n_sm*G) by (B*-1, g position); +inf padding. Rows of 17 words, so that a
-    // warp reading one g position of 32 rows (lane = row) touches 32 distinct banks.
-    float ipar[kMaxB][kIparStride];
-    float rcp[8];                    // 1 / IPC per class
-    float rcpn[33];                  // 1 / n for n = 1..32 (axis-subset sizes; [0] unused)
-    float hide[kMaxW + 1];           // max(1, W_sat / W*)
-    float lane[32];                  // (32 * W_B) / T by t position
-    int wb[32];                      // W_B = ceil(T / 32) by t position
-    int gw[32];                      // G_W by t position (0 if T > max threads per block)
-    unsigned char divt[kMaxW + 1][32];  // floor(w / W_B) by (w, t position)
-    unsigned char perm[kMaxB][16];   // g positions of ipar row b in increasing (value, g) order
-    float iparmin[kMaxB];            // min of ipar row b over all axis grid sizes
-    unsigned short rwarps[256];      // register-limited warps by R (Eq. 4, per-warp allocation)
-    unsigned short rwbmax[256];      // largest W_B whose block fits the per-block register limit, by R
-    int cap_lo[4];                   // first capacity index allowed by carveout position c
-    int order_safe;                  // 1: distinct ipar values of a row differ by more than 2^-21 relative
-    int unit_shift;                  // log2 of the shared-memory allocation unit, or -1
-};
 
 // Parameters of one launch. The CTA tables depend on the architecture row and the axes only, so the host
 // builds them and passes them here, 6.6 KB of kernel parameters each CTA copies to shared memory.
@@ -113,159 +89,6 @@ struct WarpTables {
         };
     };
 };
-
-// The tables of an architecture row and axes (IEEE single-precision divisions and multiplications, each
-// rounded to nearest as __fdiv_rn / __fmul_rn round them on the device).
-void host_cta_tables(const tune_arch& a, const tune_axes& x, CtaTables& ct)
-{
-    memset(&ct, 0, sizeof(ct));
-    const float inf = std::numeric_limits<float>::infinity();
-    for (int b = 0; b < kMaxB; ++b)
-        for (int g = 0; g < 16; ++g) {
-            float v = inf;
-            if (b < a.max_blocks_sm && g < x.n_g) {
-                const int slots = a.n_sm * (b + 1), G = x.g[g];
-                const int waves = (G + slots - 1) / slots;
-                v = (float)(waves * slots) / (float)(a.n_sm * G);
-            }
-            ct.ipar[b][g] = v;
-        }
-    for (int w = 0; w <= kMaxW; ++w)
-        for (int t = 0; t < 32; ++t) {
-            const int wb = t < x.n_t ? (x.t[t] + 31) / 32 : 1;
-            ct.divt[w][t] = (unsigned char)(w / wb);
-        }
-    // With distinct ipar values more than 2^-21 apart, X * v keeps their order strictly for every X > 0 (no
-    // underflow), so a walk in perm order meets equal costs only from equal values, in increasing g (and index)
-    // order.
-    ct.order_safe = 1;
-    const int u = a.smem_alloc_unit;
-    ct.unit_shift = (u & (u - 1)) == 0 ? __builtin_ctz((unsigned)u) : -1;
-    for (int b = 0; b < kMaxB; ++b) {
-        float mn = inf;
-        for (int g = 0; g < x.n_g; ++g) mn = std::min(mn, ct.ipar[b][g]);
-        ct.iparmin[b] = mn;
-        unsigned char* ord = ct.perm[b];
-        for (int g = 0; g < x.n_g; ++g) {
-            const float v = ct.ipar[b][g];
-            int j = g;
-            while (j > 0 && ct.ipar[b][ord[j - 1]] > v) {
-                ord[j] = ord[j - 1];
-                --j;
-            }
-            ord[j] = (unsigned char)g;
-        }
-        for (int r = 0; r + 1 < x.n_g; ++r) {
-            const float v1 = ct.ipar[b][ord[r]], v2 = ct.ipar[b][ord[r + 1]];
-            const volatile float gap = v2 - v1, tol = v1 * 0x1p-21f;  // two roundings, no fused form
-            if (v2 != v1 && gap <= tol) ct.order_safe = 0;
-        }
-    }
-    for (int t = 0; t < 32; ++t) {
-        int wb = 1, gw = 0;
-        float ln = 1.0f;
-        if (t < x.n_t) {
-            const int T = x.t[t];
-            wb = (T + 31) / 32;
-            gw = T <= a.max_threads_block ? std::min(a.max_blocks_sm, a.max_warps_sm / wb) : 0;
-            ln = (float)(32 * wb) / (float)T;
-        }
-        ct.wb[t] = wb;
-        ct.gw[t] = gw;
-        ct.lane[t] = ln;
-    }
-    for (int w = 0; w <= kMaxW; ++w) ct.hide[w] = std::max(1.0f, w > 0 ? (float)a.w_sat / (float)w : 1.0f);
-    for (int c = 0; c < 8; ++c) ct.rcp[c] = c < TUNE_NCLASS ? 1.0f / a.ipc[c] : 0.0f;
-    for (int n = 1; n <= 32; ++n) ct.rcpn[n] = 1.0f / (float)n;
-    for (int c = 0; c < 4; ++c) {
-        const long long need = c < x.n_c ? (long long)x.c[c] * a.smem_caps[a.n_smem_caps - 1] : 0;
-        int i = 0;
-        while (i < a.n_smem_caps && 100LL * a.smem_caps[i] < need) ++i;
-        ct.cap_lo[c] = i;
-    }
-    for (int R = 0; R < 256; ++R) {
-        int warps, wbmax;
-        reg_params(a, R, warps, wbmax);
-        ct.rwarps[R] = (unsigned short)warps;
-        ct.rwbmax[R] = (unsigned short)std::min(wbmax, 65535);
-    }
-}
-
-// host_cta_tables for the launch, from the calling thread's last kMaxArch different rows and axes where they are
-// among them (compared byte for byte).
-void fill_host_tables(EvalParams& q)
-{
-    struct Entry {
-        tune_arch a;
-        tune_axes x;
-        CtaTables t;
-    };
-    static thread_local Entry kept[kMaxArch];
-    static thread_local int n_kept = 0, oldest = 0;
-    for (int i = 0; i < n_kept; ++i)
-        if (memcmp(&kept[i].a, &q.a, sizeof(tune_arch)) == 0 && memcmp(&kept[i].x, &q.x, sizeof(tune_axes)) == 0) {
-            q.tab = kept[i].t;
-            return;
-        }
-    Entry& e = kept[n_kept < kMaxArch ? n_kept++ : (oldest++ % kMaxArch)];
-    e.a = q.a;
-    e.x = q.x;
-    host_cta_tables(e.a, e.x, e.t);
-    q.tab = e.t;
-}
-
-// The tables from the launch parameters into shared memory (a word per thread and step).
-__device__ __forceinline__ void copy_cta_tables(const CtaTables& src, CtaTables& ct)
-{
-    const uint32_t* s = reinterpret_cast<const uint32_t*>(&src);
-    uint32_t* d = reinterpret_cast<uint32_t*>(&ct);
-    for (int i = threadIdx.x; i < (int)(sizeof(CtaTables) / 4); i += blockDim.x) d[i] = s[i];
-}
-
-// q = floor(n / d) for 0 <= n < 2^25 and 1 <= d < 2^25: a single-precision estimate
-// (within 2 of q) corrected with exact integer remainders.
-__device__ __forceinline__ int udiv_small(int n, int d)
-{
-    int q = __float2int_rz(__fmul_rn((float)n, __frcp_rn((float)d)));
-    int r = n - q * d;
-    while (r < 0) {
-        --q;
-        r += d;
-    }
-    while (r >= d) {
-        ++q;
-        r -= d;
-    }
-    return q;
-}
-
-// G_S (Eq. 5) as smem_blocks(), starting the capacity search at the carveout's
-// first admissible capacity (carveout position cp).
-__device__ __forceinline__ int smem_blocks_from(const tune_arch& a, const CtaTables& ct, int s0, int cp)
-{
-    if (s0 > a.smem_block_max) return 0;
-    const int need = s0 + a.smem_reserved_block;
-    const int unit = a.smem_alloc_unit;
-    const int s_alloc = ct.unit_shift >= 0 ? ((need + unit - 1) >> ct.unit_shift) << ct.unit_shift
-                                           : ceil_div(need, unit) * unit;
-    if (s_alloc == 0) return a.max_blocks_sm;
-    for (int i = ct.cap_lo[cp]; i < a.n_smem_caps; ++i) {
-        const int ci = a.smem_caps[i];
-        if (ci >= s_alloc) return udiv_small(ci, s_alloc);
-    }
-    return 0;
-}
-
-// G_R (Eq. 4) for R registers and blocks of W_B warps (t position tp).
-__device__ __forceinline__ int reg_blocks(const tune_arch& a, const CtaTables& ct, int R, int wb, int tp,
-                                          int warps, int wbmax)
-{
-    if (R > a.regs_thread_max) return 0;
-    if (R <= 0) return a.max_blocks_sm;
-    if (a.reg_alloc_mode == 0) return wb > wbmax ? 0 : ct.divt[warps][tp];
-    const long long rpb = (long long)ceil_div(R * 32 * wb, a.reg_alloc_unit) * a.reg_alloc_unit;
-    return rpb > a.regs_block_max ? 0 : (int)(a.regs_sm / rpb);
-}
 
 // Sorted insert of (c, i) into a lane's register list (ascending; strict "<"
 // keeps earlier = lower-index entries first among equal costs).
@@ -1193,7 +1016,7 @@ int launch_thread(const EvalParams& p, const tune_kernel_desc* descs, int32_t* t
     const int64_t cap = (int64_t)sms * per_sm;
     const int grid = (int)(need < cap ? need : cap);
     EvalParams q = p;
-    fill_host_tables(q);
+    tune::eval_tables(q.a, q.x, q.tab);
     kern<<<grid, kThreadsT, 0, s>>>(q, reinterpret_cast<const int4*>(descs), ti, tc, status);
     TUNE_CUDA_TRY(cudaGetLastError(), "tune_eval: kernel launch");
     return TUNE_OK;
@@ -1221,7 +1044,7 @@ int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, floa
     // emitting: as many descriptors at a time, up to one per warp, as leave each CTA about three turns (the queue
     // evens out spaces of different sizes)
     q.group = (int)std::max<int64_t>(1, std::min<int64_t>(kWarps, p.n_kernels / (3 * cap)));
-    fill_host_tables(q);
+    tune::eval_tables(q.a, q.x, q.tab);
     const int4* d = reinterpret_cast<const int4*>(descs);
     if (dependent)
         TUNE_CUDA_TRY(pdl::launch_dep(kern, dim3(grid), dim3(kThreads), 0, s, q, d, ti, tc, pb, pw, pc, po, status, queue),
