@@ -373,7 +373,7 @@ int tune_emit_count(const tune_axes* axes, const tune_kernel_desc* descs, int64_
 
 /*
  * tune_eval_archs — tune_eval of the same descriptors against n_arch
- * architecture rows (1..8) in one launch (a sweep over GPU generations:
+ * architecture rows (1..8) in one call (a sweep over GPU generations:
  * Eqs. 1-6 with each row's limits and throughputs). archs: host array
  * [n_arch]. Outputs topk_idx / topk_cost [n_arch][n_kernels][k]; row i's
  * results equal tune_eval(&archs[i], ...) bit for bit. flags: TUNE_SCHED_WARP

@@ -24,13 +24,18 @@ def _torch():
 
 
 def _stream(stream):
+    """The stream's handle as an integer (the current device's current stream if None)."""
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    # (the handle without a Stream object around it: 0.2 us instead of 3 per call)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def tune_workspace_bytes(call, n, k):
@@ -80,7 +85,7 @@ def tune_eval(arch, axes, descs, k, flags=0, topk_idx=None, topk_cost=None, pt_b
 
 
 def tune_eval_archs(archs, axes, descs, k, flags=0, workspace_buf=None, stream=None):
-    """tune_eval against several architecture rows in one launch.
+    """tune_eval against several architecture rows in one call.
     Returns (topk_idx int32 [n_arch, n, k], topk_cost float32 [n_arch, n, k])."""
     torch = _torch()
     L = native.load()

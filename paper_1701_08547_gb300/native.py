@@ -7,6 +7,7 @@ other code path.
 """
 
 import ctypes as C
+import operator
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -110,8 +111,7 @@ TUNE_SEARCH_RANDOM, TUNE_SEARCH_NELDER_MEAD = 1, 2
 TUNE_REAL_MATVEC, TUNE_REAL_ATAX, TUNE_REAL_BICG = 0, 1, 2
 
 
-def make_arch(row):
-    """Marshal an architecture-row dict into the C struct."""
+def _make_arch_each(row):
     a = TuneArch()
     for f, _ in TuneArch._fields_:
         if f in ("smem_caps", "ipc"):
@@ -127,8 +127,7 @@ def make_arch(row):
     return a
 
 
-def make_axes(ax):
-    """Marshal an axes dict {t, g, u, c: lists} into the C struct."""
+def _make_axes_each(ax):
     a = TuneAxes()
     a.n_t, a.n_g, a.n_u, a.n_c = len(ax["t"]), len(ax["g"]), len(ax["u"]), len(ax["c"])
     for name in ("t", "g", "u", "c"):
@@ -136,6 +135,33 @@ def make_axes(ax):
         for i, v in enumerate(ax[name]):
             arr[i] = int(v)
     return a
+
+
+_ARCH_INTS = operator.itemgetter(*[f for f, _ in TuneArch._fields_[:15]])
+
+
+def make_arch(row):
+    """Marshal an architecture-row dict into the C struct."""
+    try:  # whole arrays at once where the values are plain numbers of the fields' kinds
+        caps, ipc = row["smem_caps"], row["ipc"]
+        a = TuneArch(*_ARCH_INTS(row), len(caps))
+        a.smem_caps[:len(caps)] = caps
+        a.ipc[:len(ipc)] = ipc
+        a.w_sat, a.work_scale = row["w_sat"], row["work_scale"]
+        return a
+    except (TypeError, ValueError, IndexError):
+        return _make_arch_each(row)
+
+
+def make_axes(ax):
+    """Marshal an axes dict {t, g, u, c: lists} into the C struct."""
+    try:
+        t, g, u, c = ax["t"], ax["g"], ax["u"], ax["c"]
+        a = TuneAxes(len(t), len(g), len(u), len(c))
+        a.t[:len(t)], a.g[:len(g)], a.u[:len(u)], a.c[:len(c)] = t, g, u, c
+        return a
+    except (TypeError, ValueError, IndexError):
+        return _make_axes_each(ax)
 
 
 def check(rc):

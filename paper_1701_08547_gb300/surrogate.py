@@ -2,7 +2,7 @@
 
 import ctypes as C
 
-from . import native
+from . import _ptr, _stream, native
 
 
 class Cfg(C.Structure):
@@ -41,13 +41,6 @@ def _lib():
         L.surrogate_status.restype = C.c_int
         L._surrogate_declared = True
     return L
-
-
-def _stream(stream):
-    import torch
-
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
 
 
 class Surrogate:
@@ -120,23 +113,18 @@ class Surrogate:
         n = feats.shape[0]
         if pred is None:
             pred = torch.empty((self.members, n), dtype=torch.float32, device=feats.device)
-        native.check(self.L.surrogate_forward(self.h, C.c_void_p(feats.data_ptr()), n,
-                                              C.c_void_p(pred.data_ptr()), _stream(stream)))
+        native.check(self.L.surrogate_forward(self.h, _ptr(feats), n, _ptr(pred), _stream(stream)))
         return pred
 
     def train_step(self, feats, labels, apply_update=True, stream=None):
         n = feats.shape[0]
-        native.check(self.L.surrogate_train_step(self.h, C.c_void_p(feats.data_ptr()),
-                                                 C.c_void_p(labels.data_ptr()), n, int(apply_update),
+        native.check(self.L.surrogate_train_step(self.h, _ptr(feats), _ptr(labels), n, int(apply_update),
                                                  _stream(stream)))
 
     def train(self, feats, labels, order, epochs, loss_trace=None, stream=None):
         n = feats.shape[0]
-        lt = None if loss_trace is None else C.c_void_p(loss_trace.data_ptr())
-        native.check(self.L.surrogate_train(self.h, C.c_void_p(feats.data_ptr()),
-                                            C.c_void_p(labels.data_ptr()), n,
-                                            C.c_void_p(order.data_ptr()), int(epochs), lt,
-                                            _stream(stream)))
+        native.check(self.L.surrogate_train(self.h, _ptr(feats), _ptr(labels), n, _ptr(order), int(epochs),
+                                            _ptr(loss_trace), _stream(stream)))
 
     def infer(self, arch, axes, descs, pt_offsets, k, thresh=0.1, stream=None):
         """Rank every point of every kernel by predicted runtime with analytic fallback.
@@ -154,8 +142,7 @@ class Surrogate:
         nbytes = self.L.surrogate_infer_workspace_bytes(self.members, n, k)
         ws = torch.empty(nbytes, dtype=torch.uint8, device=dev)
         a, x = native.make_arch(arch), native.make_axes(axes)
-        native.check(self.L.surrogate_infer(self.h, C.byref(a), C.byref(x), C.c_void_p(descs.data_ptr()), n,
-                                            off.ctypes.data, int(k), float(thresh), C.c_void_p(idx.data_ptr()),
-                                            C.c_void_p(val.data_ptr()), C.c_void_p(fb.data_ptr()),
-                                            C.c_void_p(ws.data_ptr()), nbytes, _stream(stream)))
+        native.check(self.L.surrogate_infer(self.h, C.byref(a), C.byref(x), _ptr(descs), n,
+                                            off.ctypes.data, int(k), float(thresh), _ptr(idx), _ptr(val), _ptr(fb),
+                                            _ptr(ws), nbytes, _stream(stream)))
         return idx, val, fb
