@@ -19,6 +19,11 @@
 // inputs (the MN-major 128-byte-swizzle atoms, 8 KB apart along N), from the same BF16
 // copy the forward pass uses.
 //
+// Bound by the chain of a unit (three products, each after the epilogue before it) and, since 320
+// units of 8,192 rows x 5 members leave 16 of 152 CTAs a third, lone unit, by that unit's latency.
+// 14 training steps 2.06 -> 2.05 ms with the issuing warp converged (its descriptors in uniform
+// registers, one elected lane issuing), 32-bit unit numbers and one arrival per epilogue warp.
+//
 // Every wait is bounded; on timeout the kernel sets status bit 2, stops issuing
 // work, waits (bounded) for the copies and MMAs it issued, frees its tensor memory
 // and returns.
@@ -51,6 +56,15 @@ struct BwdArgs {
 };
 
 
+// A persistent CTA's unit of ordinal jj (units < 2^28, so 32-bit division), the last tile first: the
+// weight gradients read the batch from its first tile, whose dZ are then the latest written.
+__device__ __forceinline__ Unit bwd_unit(int jj, int units, int members)
+{
+    const unsigned u = (unsigned)max(units - 1 - ((int)blockIdx.x + jj * (int)gridDim.x), 0);
+    const unsigned t = u / (unsigned)members;
+    return {(int)t, (int)(u - t * (unsigned)members)};
+}
+
 // grid: min(SMs, units) persistent CTAs; CTA b runs units b, b + gridDim.x, ...; its
 // j-th unit goes to chain j % 2. Unit u = (tile u / members, member u % members).
 // tdz: dZ4 as 8-byte elements {64, rows, members}, box {16, 128, 1};
@@ -71,8 +85,9 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* ring = smem + 2 * C::act_bytes;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long my_units = g.units > (long long)blockIdx.x ? (g.units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int units = (int)g.units;
+    const int my_units = units > (int)blockIdx.x ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     volatile int* abort_v = &abort_flag;
 
     pdl::grid_dep_enter();  // launched after the head backward in a training step
@@ -90,7 +105,7 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
             tc::mbar_init(&x_full[s], 1);
             tc::mbar_init(&act_free[s], 1);
             tc::mbar_init(&acc_full[s], 1);
-            tc::mbar_init(&act_ready[s], 32 * kEpiWarps);
+            tc::mbar_init(&act_ready[s], kEpiWarps);
         }
         tc::mbar_init(&drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -104,16 +119,17 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
     if (warp == 0) {
         // ---- producer: per unit pair, stage by stage, chain by chain (the MMA order) ----
         if (lane == 0) {
-            long long seq = 0;
-            long long x_last[2] = {-1, -1};
+            const uint64_t g_policy = policy_evict_first();  // read once, below
+            int seq = 0;
+            int x_last[2] = {-1, -1};
             bool ok = true;
-            for (long long j = 0; j < my_units && ok; j += 2) {
+            for (int j = 0; j < my_units && ok; j += 2) {
+                const Unit un[2] = {bwd_unit(j, units, g.members), bwd_unit(j + 1, units, g.members)};
                 for (int l = 0; l < kBwdStages && ok; ++l) {
                     for (int s = 0; s < 2 && ok; ++s) {
-                        const long long jj = j + s;
+                        const int jj = j + s;
                         if (jj >= my_units) break;
-                        const long long u = blockIdx.x + jj * gridDim.x;
-                        const int tile = (int)(u / g.members), mem = (int)(u % g.members);
+                        const int tile = s ? un[1].tile : un[0].tile, mem = s ? un[1].mem : un[0].mem;
                         if (l == 0) {
                             if (jj >= 2 && !(ok = wait_bar(&act_free[s], (uint32_t)(((jj - 2) >> 1) & 1), g.status,
                                                            abort_v)))
@@ -130,13 +146,14 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
                             const char* gt = reinterpret_cast<const char*>(
                                 g.g[l] + (long long)mem * g.act_stride + (long long)tile * kRows * kWid);
                             for (int q = 0; q < 2; ++q)
-                                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(gt + q * 32768),
-                                             "r"(32768)
+                                asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;\n" ::"l"(
+                                                 gt + q * 32768),
+                                             "r"(32768), "l"(g_policy)
                                              : "memory");
                         }
                         for (int c = 0; c < kChunks; ++c, ++seq) {
-                            const int st = (int)(seq % C::stages);
-                            const long long use = seq / C::stages;
+                            const int st = seq % C::stages;
+                            const int use = seq / C::stages;
                             if (use > 0 && !(ok = wait_bar(&w_empty[st], (uint32_t)((use - 1) & 1), g.status,
                                                            abort_v)))
                                 break;
@@ -151,7 +168,7 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
                 }
             }
             if (!ok) {
-                for (long long q = seq - C::stages; q < seq; ++q)
+                for (int q = seq - C::stages; q < seq; ++q)
                     if (q >= 0)
                         tc::mbar_wait(&w_full[q % C::stages], (uint32_t)((q / C::stages) & 1), g.status);
                 for (int s = 0; s < 2; ++s)
@@ -159,59 +176,71 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
             }
         }
     } else if (warp == 1) {
-        // ---- MMA issuer ----
-        if (lane == 0) {
-            long long seq = 0;
-            bool ok = true;
-            // A (the dZ rows) K-major, B (W as stored) MN-major
-            const uint32_t idesc = tc::idesc_bf16(kRows, kWid) | (1u << 16);
-            for (long long j = 0; j < my_units && ok; j += 2) {
-                for (int l = 0; l < kBwdStages && ok; ++l) {
-                    for (int s = 0; s < 2 && ok; ++s) {
-                        const long long jj = j + s;
-                        if (jj >= my_units) break;
-                        const long long k = jj >> 1;
-                        if (l == 0 && !(ok = wait_bar(&x_full[s], (uint32_t)(k & 1), g.status, abort_v))) break;
-                        // the chain's previous epilogue has written act and drained acc
-                        const long long ph = kBwdStages * k + l - 1;
-                        if (ph >= 0 && !(ok = wait_bar(&act_ready[s], (uint32_t)(ph & 1), g.status, abort_v)))
-                            break;
+        // ---- MMA issuer: the whole warp walks the loop (uniform descriptors and waits), one elected
+        // lane issues ----
+        const bool leader = elect_one();
+        int st = 0;
+        uint32_t wph = 0;
+        bool ok = true;
+        // A (the dZ rows) K-major, B (W as stored) MN-major
+        const uint32_t idesc = tc::idesc_bf16(kRows, kWid) | (1u << 16);
+        const uint64_t b_ring = sdesc_w_mn(ring);
+        for (int j = 0; j < my_units && ok; j += 2) {
+            const Unit un[2] = {bwd_unit(j, units, g.members), bwd_unit(j + 1, units, g.members)};
+            const int ns = min(2, my_units - j);
+            const uint32_t k = (uint32_t)(j >> 1);
+            for (int l = 0; l < kBwdStages && ok; ++l) {
+#pragma unroll 1
+                for (int s = 0; s < ns && ok; ++s) {
+                    if (l == 0 && !(ok = wait_bar_warp(&x_full[s], k & 1, g.status, abort_v))) break;
+                    // the chain's previous epilogue has written act and drained acc
+                    const int ph = kBwdStages * (int)k + l - 1;
+                    if (ph >= 0 && !(ok = wait_bar_warp(&act_ready[s], (uint32_t)(ph & 1), g.status, abort_v))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const uint8_t* act = smem + s * C::act_bytes;
+                    if (l > 0 && leader) {
+                        // act holds the previous stage's dZ (this unit's rows): copied to global
+                        // memory by the tensor-store unit while the MMAs below read it
+                        for (int c = 0; c < kChunks; ++c)
+                            tma_store_4d(&tdzs, act + c * kChunkA, c * 16, (s ? un[1].tile : un[0].tile) * kRows,
+                                         s ? un[1].mem : un[0].mem, g.dz_coord[l - 1]);
+                        bulk_commit();
+                    }
+                    const uint32_t d = tmem + (uint32_t)(s * kWid);
+                    uint64_t a = tc::sdesc(act);  // addresses in the descriptors count 16-byte units
+                    for (int c = 0; c < kChunks; ++c, a += kChunkA >> 4) {
+                        if (!(ok = wait_bar_warp(&w_full[st], wph, g.status, abort_v))) break;
                         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        const uint8_t* act = smem + s * C::act_bytes;
-                        if (l > 0) {
-                            // act holds the previous stage's dZ (this unit's rows): copied to global
-                            // memory by the tensor-store unit while the MMAs below read it
-                            const long long u = blockIdx.x + jj * gridDim.x;
-                            const int tile = (int)(u / g.members), mem = (int)(u % g.members);
-                            for (int c = 0; c < kChunks; ++c)
-                                tma_store_4d(&tdzs, act + c * kChunkA, c * 16, tile * kRows, mem, g.dz_coord[l - 1]);
-                            bulk_commit();
-                        }
-                        const uint32_t d = tmem + (uint32_t)(s * kWid);
-                        for (int c = 0; c < kChunks; ++c, ++seq) {
-                            const int st = (int)(seq % C::stages);
-                            if (!(ok = wait_bar(&w_full[st], (uint32_t)((seq / C::stages) & 1), g.status, abort_v)))
-                                break;
-                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        const uint64_t b = b_ring + (uint64_t)(st * (kChunkW >> 4));
+                        if (leader) {
 #pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {
-                                const uint64_t a = tc::sdesc(act + c * kChunkA + kk * 32);
-                                const uint64_t b = sdesc_w_mn(ring + st * kChunkW + kk * 2048);
-                                tc::mma_bf16(d, a, b, idesc, (c | kk) != 0);
-                            }
+                            for (int kk = 0; kk < 4; ++kk)
+                                tc::mma_bf16(d, a + kk * 2, b + kk * (2048 >> 4), idesc, (c | kk) != 0);
                             tc::mma_commit(&w_empty[st]);
                         }
-                        if (l > 0) bulk_wait_read();  // the epilogue rewrites act after acc_full
-                        if (!ok) break;
-                        tc::mma_commit(&acc_full[s]);
-                        if (l == kBwdStages - 1) tc::mma_commit(&act_free[s]);
+                        __syncwarp();
+                        if (++st == C::stages) {
+                            st = 0;
+                            wph ^= 1;
+                        }
                     }
+                    if (leader) {
+                        if (l > 0) bulk_wait_read();  // the epilogue rewrites act after acc_full
+                        if (ok) {
+                            tc::mma_commit(&acc_full[s]);
+                            if (l == kBwdStages - 1) tc::mma_commit(&act_free[s]);
+                        }
+                    }
+                    __syncwarp();
                 }
             }
+        }
+        if (leader) {
             bulk_wait_all();
             tc::mma_commit(&drain);
             tc::mbar_wait(&drain, 0, g.status);
         }
+        __syncwarp();
     } else {
         // ---- epilogue: dZ = bf16(acc * gelu'(z)) to global memory and, before the last
         // stage, to the chain's activation buffer as the next product's A operand ----
@@ -219,15 +248,13 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
         const int r = q * 32 + lane;
         const int c_beg = cq * (kWid / 4);
         bool ok = true;
-        for (long long j = 0; j < my_units && ok; j += 2) {
+        for (int j = 0; j < my_units && ok; j += 2) {
+            const Unit u0 = bwd_unit(j, units, g.members), u1 = bwd_unit(j + 1, units, g.members);
+            const int ns = min(2, my_units - j), k = j >> 1;
             for (int l = 0; l < kBwdStages && ok; ++l) {
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    const long long jj = j + s;
-                    if (jj >= my_units || !ok) break;
-                    const long long k = jj >> 1;
-                    const long long u = blockIdx.x + jj * gridDim.x;
-                    const int tile = (int)(u / g.members), mem = (int)(u % g.members);
+#pragma unroll 1
+                for (int s = 0; s < ns; ++s) {
+                    const int tile = s ? u1.tile : u0.tile, mem = s ? u1.mem : u0.mem;
                     const int row = tile * kRows + r;
                     const long long arow = (long long)mem * g.act_stride + (long long)row * kWid;
                     const __half* gr = g.g[l] + (long long)mem * g.act_stride;  // tiled (mlp::gprime_at)
@@ -240,8 +267,7 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
                     uint32_t gw[kWid / 4 / 16][8];
 #pragma unroll
                     for (int b = 0; b < kWid / 4 / 16; ++b) ld_global_v8u(gr + mlp::gprime_at(row, c_beg + 16 * b), gw[b]);
-                    if (!(ok = wait_bar(&acc_full[s], (uint32_t)((kBwdStages * k + l) & 1), g.status, abort_v)))
-                        break;
+                    if (!(ok = wait_bar_warp(&acc_full[s], (uint32_t)((kBwdStages * k + l) & 1), g.status, abort_v))) break;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
                     for (int b = 0; b < kWid / 4 / 16; ++b) {
@@ -266,7 +292,8 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
                     }
                     if (!last) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                    mbar_arrive(&act_ready[s]);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&act_ready[s]);
                 }
             }
         }

@@ -8,7 +8,8 @@
 // long a unit takes by itself: sixteen warps serve each unit's epilogue, load their columns of the
 // accumulator at once (which frees it for the next layer) and hand the layer's output over one K chunk at a
 // time, so that the next layer's MMAs start while the later chunks are still being computed. 14 steps of
-// 8,192 rows x 5 members: 2.17 -> 2.05 ms (2.21 with the inference kernel's split of the warps).
+// 8,192 rows x 5 members: 2.17 -> 2.05 ms (2.21 with the inference kernel's split of the warps);
+// 1.89 ms with the backward kernels' changes and the L2 policies (policy_evict_first).
 #pragma once
 
 #include "tc_mlp.cuh"
@@ -252,6 +253,7 @@ __global__ void __maxnreg__(96) mlp_train_kernel(const __grid_constant__ CUtenso
         uint32_t wph = 0;
         bool ok = true;
         const uint64_t b_ring = tc::sdesc(ring);
+        const uint64_t h_policy = policy_evict_first();  // H1..H3 are read last of all, by the weight gradients
         for (int j = 0; j < my_units && ok; j += 2) {
             const Unit un[2] = {train_unit(j, g.members), train_unit(j + 1, g.members)};
             const int ns = min(2, my_units - j);
@@ -285,7 +287,7 @@ __global__ void __maxnreg__(96) mlp_train_kernel(const __grid_constant__ CUtenso
                             // by the tensor-store unit while the MMAs read it
                             if (l > 0)
                                 tma_store_4d(&th, act + c * kChunkA, c * 16, (s ? un[1].tile : un[0].tile) * kRows,
-                                             s ? un[1].mem : un[0].mem, l - 1);
+                                             s ? un[1].mem : un[0].mem, l - 1, h_policy);
                         }
                         __syncwarp();
                         if (++st == C::stages) {

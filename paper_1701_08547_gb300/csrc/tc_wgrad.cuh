@@ -27,6 +27,11 @@
 // stages, warp 1 issues the MMAs, warps 2-5 read the accumulator back (thread = output
 // row, one warp per TMEM lane quarter) and store the gradient rows.
 //
+// Bound by reading dZ and H: 8,192 rows x 5 members are 168 MB, most of it from DRAM (146 MB of reads
+// in 35 us with no L2 policies; tcm::policy_evict_first). 14 training steps 2.06 -> 2.05 ms with the
+// issuing warp converged, 2.03 with the barriers and the all-ones block set up before the wait for
+// the launch before (136 SMs are free while the last units of the input-gradient chain run).
+//
 // Every wait is bounded; on timeout the kernel sets status bit 2, stops issuing work,
 // waits (bounded) for the copies and MMAs it issued, frees its tensor memory and returns.
 #pragma once
@@ -104,9 +109,8 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constan
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* ones = smem + kStages * kStage;  // 1 KB aligned, after every stage
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int mem = blockIdx.y;
-    pdl::grid_dep_enter();  // launched after the input-gradient chain in a training step
     // tile -> (layer item j, output half, input column block)
     int j = 0, tt = blockIdx.x;
     while (j < g.n_items && tt >= 2 * (g.kin[j] / kTileCols)) {
@@ -120,11 +124,6 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constan
     const int n = g.chunks;
     volatile int* abort_v = &abort_flag;
 
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tc::sa(&tmem_base)),
-                     "r"(kTmemCols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-    }
     if (threadIdx.x == 32) {
         for (int i = 0; i < kStages; ++i) {
             tc::mbar_init(&full[i], 1);
@@ -138,6 +137,12 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constan
     // the all-ones block (BF16 1.0 = 0x3f80), made visible to the tensor cores' proxy
     for (int i = threadIdx.x; i < kOnes / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(ones)[i] = 0x3f803f80u;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    pdl::grid_dep_enter();  // launched after the input-gradient chain in a training step
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tc::sa(&tmem_base)),
+                     "r"(kTmemCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -146,6 +151,8 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constan
     if (warp == 0) {
         // ---- producer ----
         if (lane == 0 && n > 0) {
+            // dZ and Hprev are read by the CTAs of this launch, at about the same time, and not again
+            const uint64_t policy = tcm::policy_evict_first();
             int i = 0;
             bool ok = true;
             for (; i < n; ++i) {
@@ -155,33 +162,49 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_kernel(const __grid_constan
                 const int r0 = i * kChunkRows;
                 tc::mbar_expect_tx(&full[st], (uint32_t)kStage);
                 for (int q = 0; q < 2; ++q)
-                    tc::tma_load_3d(a + q * kBox, &maps.ta[j], (2 * half + q) * 16, r0, mem, &full[st]);
-                tc::tma_load_3d(a + kStageA, &maps.tb[j], cb * 16, r0, g.b_batched[j] ? mem : 0, &full[st]);
+                    tcm::tma_load_3d(a + q * kBox, &maps.ta[j], (2 * half + q) * 16, r0, mem, &full[st], policy);
+                tcm::tma_load_3d(a + kStageA, &maps.tb[j], cb * 16, r0, g.b_batched[j] ? mem : 0, &full[st], policy);
             }
             if (!ok)  // let the copies in flight land before the CTA exits
                 for (int q = i - kStages; q < i; ++q)
                     if (q >= 0) tc::mbar_wait(&full[q % kStages], (uint32_t)((q / kStages) & 1), g.status);
         }
     } else if (warp == 1) {
-        // ---- MMA issuer ----
-        if (lane == 0 && n > 0) {
+        // ---- MMA issuer: the whole warp walks the loop (uniform descriptors and waits), one elected
+        // lane issues ----
+        if (n > 0) {
+            const bool leader = tcm::elect_one();
             // bias tiles: N = 64 Hprev columns + 16 all-ones columns (the atom at ones)
             const uint32_t idesc = idesc_bf16_mn(128, bias ? kTileCols + kBiasCols : kTileCols);
+            const uint64_t a0 = sdesc_mn(smem), b0 = sdesc_mn(smem + kStageA, (uint32_t)(ones - (smem + kStageA)));
+            int st = 0;
+            uint32_t ph = 0;
             bool ok = true;
-            for (int i = 0; i < n && ok; ++i) {
-                const int st = i % kStages;
-                if (!(ok = tcm::wait_bar(&full[st], (uint32_t)((i / kStages) & 1), g.status, abort_v))) break;
+            for (int i = 0; i < n; ++i) {
+                if (!(ok = tcm::wait_bar_warp(&full[st], ph, g.status, abort_v))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint8_t* a = smem + st * kStage;
+                // stage st: addresses (16-byte units) up, the distance to the ones block down by st stages
+                const uint64_t a = a0 + (uint64_t)(st * (kStage >> 4));
+                const uint64_t b = b0 + (uint64_t)(st * (kStage >> 4)) - ((uint64_t)(st * (kStage >> 4)) << 16);
+                if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < kChunkRows / 16; ++kk)  // 16 batch rows = two K atoms per step
-                    tc::mma_bf16(tmem, sdesc_mn(a + kk * 2048),
-                                 sdesc_mn(a + kStageA + kk * 2048, (uint32_t)(ones - (a + kStageA))), idesc, (i | kk) != 0);
-                tc::mma_commit(&empty[st]);
+                    for (int kk = 0; kk < kChunkRows / 16; ++kk)  // 16 batch rows = two K atoms per step
+                        tc::mma_bf16(tmem, a + kk * (2048 >> 4),
+                                     b + kk * (2048 >> 4), idesc, (i | kk) != 0);
+                    tc::mma_commit(&empty[st]);
+                }
+                __syncwarp();
+                if (++st == kStages) {
+                    st = 0;
+                    ph ^= 1;
+                }
             }
-            if (ok) tc::mma_commit(&acc_full);
-            tc::mma_commit(&drain);  // arrives when every MMA issued above has completed
-            tc::mbar_wait(&drain, 0, g.status);
+            if (leader) {
+                if (ok) tc::mma_commit(&acc_full);
+                tc::mma_commit(&drain);  // arrives when every MMA issued above has completed
+                tc::mbar_wait(&drain, 0, g.status);
+            }
+            __syncwarp();
         }
     } else {
         // ---- epilogue warps ----
