@@ -8,7 +8,10 @@
 //
 // Rules that keep this correct and free of deadlock:
 //  * every kernel launched by launch_dep() calls grid_dep_wait() before any
-//    global-memory access (read or write) and before allocating tensor memory;
+//    global-memory access (read or write) and before allocating tensor memory,
+//    except reads of data that no launch from its predecessor's predecessor on
+//    writes (that one is complete when the predecessor's CTAs start their
+//    successor);
 //  * a kernel calls grid_dep_launch() only after its own grid_dep_wait(), so at
 //    most one kernel waits ahead of the running one;
 //  * in a kernel launched without the attribute both calls return at once.

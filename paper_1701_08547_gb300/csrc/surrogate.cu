@@ -133,76 +133,31 @@ __global__ void head_fwd(const __nv_bfloat16* __restrict__ H4, const float* __re
 // Column sums over rows in two stages (deterministic): stage 1 sums slices of
 // kRowSlice rows into part[mem][slice][WID + 1]; stage 2 adds the slices.
 constexpr int kRowSlice = 64;
-constexpr int kRedWarps = 32;  // warps per block of the slice sums
 
-// Loss gradient and head backward in one pass over a slice of srows rows (block = (slice,
-// member), 256 threads: eight row groups of 32 threads, each thread eight columns with 16-byte
-// accesses): dy[i] = 2 (y[i] - lbl[i]) / n for the n labelled rows (0 past them),
-// dZ4[i][j] = bf16(dy[i] * w5[j] * G4[i][j]) with G4 = gelu'(Z4), and part[.][.][j] = sum over
-// the slice of dy[i] H4[i][j] (j < 256), of dy[i] (j = 256) and of (y[i] - lbl[i])^2 (j = 257;
-// rows of kHeadStride floats). Row group q takes rows i0 + q, i0 + q + 8, ...; its sums are
-// added to the other groups' in group order.
-constexpr int kHeadGroups = 8;
-constexpr int kHeadStride = WID + 2;
+// Loss gradient and head backward in one pass over a slice of srows rows (tcm::head_rows; block = (slice,
+// member), 256 threads: eight row groups of 32 threads). Slices that the forward pass has done are
+// left out: those of units u (128-row tile u / members, member u % members) with u % fwd_grid >= fwd_first.
+// ROWS = 8 (a 64-row slice's loads all in flight) where the chip has few slices, 2 (more CTAs per SM) where it has
+// many: 14 training steps 1.85 ms against 1.87 for 96 slices a step, 1.93 against 1.89 for all 640.
+using tcm::kHeadGroups;
+using tcm::kHeadStride;
+template <int ROWS>
 __global__ void __launch_bounds__(256) head_bwd(const float* __restrict__ y, const float* __restrict__ lbl, int n,
                                                 const float* __restrict__ master, const __half* __restrict__ G4,
                                                 const __nv_bfloat16* __restrict__ H4, __nv_bfloat16* dZ, float* part,
-                                                int rows, int batch, int slices, int srows)
+                                                int rows, int batch, int slices, int srows, int fwd_grid, int fwd_first)
 {
     pdl::grid_dep_enter();  // a step of the training chain: wait for the launch before it
     __shared__ float red[kHeadGroups][kHeadStride];
     const int mem = blockIdx.y, sl = blockIdx.x;
-    const int q = threadIdx.x >> 5, j = 8 * (threadIdx.x & 31);
-    const float* yv = y + (long long)mem * batch;
-    const float n_f = (float)n;
-    const long long base = (long long)mem * batch * WID + j;
-    float w[8];
-    {
-        const float4 a = *reinterpret_cast<const float4*>(master + mem * P + OFF_W5 + j);
-        const float4 b = *reinterpret_cast<const float4*>(master + mem * P + OFF_W5 + j + 4);
-        w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
-    }
-    float sh[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, sb = 0.0f, se = 0.0f;
     const int i0 = sl * srows, i1 = min(rows, i0 + srows);
-#pragma unroll 2
-    for (int i = i0 + q; i < i1; i += kHeadGroups) {
-        float di = 0.0f;
-        if (i < n) {
-            const float e = yv[i] - lbl[i];
-            di = 2.0f * e / n_f;
-            se += e * e;
-        }
-        const long long o = base + (long long)i * WID;
-        const uint4 gv = __ldg(reinterpret_cast<const uint4*>(G4 + (long long)mem * batch * WID + mlp::gprime_at(i, j)));
-        const uint4 hv = __ldg(reinterpret_cast<const uint4*>(H4 + o));
-        const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, hw[4] = {hv.x, hv.y, hv.z, hv.w};
-        uint32_t out[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const float2 g = __half22float2(*reinterpret_cast<const __half2*>(&gw[t]));
-            const float2 h = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[t]));
-            const __nv_bfloat162 z = __floats2bfloat162_rn(di * w[2 * t] * g.x, di * w[2 * t + 1] * g.y);
-            out[t] = *reinterpret_cast<const uint32_t*>(&z);
-            sh[2 * t] = fmaf(di, h.x, sh[2 * t]);
-            sh[2 * t + 1] = fmaf(di, h.y, sh[2 * t + 1]);
-        }
-        *reinterpret_cast<uint4*>(dZ + o) = make_uint4(out[0], out[1], out[2], out[3]);
-        sb += di;
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) red[q][j + c] = sh[c];
-    if (j == 0) {
-        red[q][WID] = sb;
-        red[q][WID + 1] = se;
-    }
+    if (fwd_first < fwd_grid && (i0 / tcm::kRows * (int)gridDim.y + mem) % fwd_grid >= fwd_first) return;
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long base = (long long)mem * batch * WID;
+    tcm::head_rows<false, ROWS>(y + (long long)mem * batch, lbl, n, master + mem * P + OFF_W5, G4 + base, H4 + base, dZ + base,
+                                i0, i1, q, lane, red[q]);
     __syncthreads();
-    float* o = part + ((long long)mem * slices + sl) * kHeadStride;
-    for (int c = threadIdx.x; c < kHeadStride; c += blockDim.x) {
-        float v = red[0][c];
-#pragma unroll
-        for (int g = 1; g < kHeadGroups; ++g) v += red[g][c];
-        o[c] = v;
-    }
+    tcm::head_sum(red[0], threadIdx.x, part + ((long long)mem * slices + sl) * kHeadStride);
 }
 
 // part[.][.][j] = sum over the slice of dZ[i][j] (four independent partial sums)
@@ -221,35 +176,15 @@ __global__ void bias_partial(const __nv_bfloat16* __restrict__ dZ, float* part, 
     part[((long long)mem * slices + sl) * (WID + 1) + j] = (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// grad[mem * P + off + j] = sum over slices of part[mem][slice][j], j < cols (slice rows of
-// `stride` floats); with `loss`, column cols is the slices' sum of squared errors and
-// loss[mem] = that sum / n. Block = 32 columns x kRedWarps warps; warp w adds slices w,
-// w + kRedWarps, ... in order, then the warps' partial sums are added in warp order
-// (deterministic).
-__global__ void slices_reduce(const float* __restrict__ part, float* grad, long long off, int cols, int slices,
-                              int stride, float* loss, int n)
+// Sums of slices (tcm::reduce_task), one block per task.
+__global__ void slices_reduce(const __grid_constant__ tcm::ReduceArgs g)
 {
     pdl::grid_dep_enter();  // a step of the training chain: wait for the launch before it
-    // block = 32 columns x kRedWarps warps; warp w adds slices w, w + kRedWarps, ..., then
-    // the warps' sums are added in warp order
-    const int mem = blockIdx.y, w = threadIdx.x >> 5;
-    const int j = blockIdx.x * 32 + (threadIdx.x & 31);
-    __shared__ float red[kRedWarps][32];
-    const int ncol = cols + (loss ? 1 : 0);
-    float s = 0.0f;
-    if (j < ncol)
-        for (int q = w; q < slices; q += kRedWarps) s += part[((long long)mem * slices + q) * stride + j];
-    red[w][threadIdx.x & 31] = s;
+    __shared__ float red[tcm::kRedWarps * 32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    tcm::reduce_partial(g, blockIdx.x, w, lane, red);
     __syncthreads();
-    if (w == 0 && j < ncol) {
-        float t = red[0][threadIdx.x];
-#pragma unroll
-        for (int q = 1; q < kRedWarps; ++q) t += red[q][threadIdx.x];
-        if (j < cols)
-            grad[mem * P + off + j] = t;
-        else
-            loss[mem] = t / (float)n;
-    }
+    if (w == 0) tcm::reduce_finish(g, blockIdx.x, lane, red);
 }
 
 // grad W[o][i] = sum over splits of part[split][o][i], added in split order; four
@@ -300,20 +235,67 @@ __global__ void split_reduce(const float* __restrict__ part, float* grad, long l
     *reinterpret_cast<float4*>(grad + mem * P + off_w + e) = s;
 }
 
-// Adam on FP32 master weights, then the BF16 copies of W1..W4; four consecutive
-// parameters per thread (every parameter segment starts at a multiple of 4, so a group
-// lies in one segment; padding past the last parameter is left alone).
-__global__ void adam_update(float* master, const float* grad, float* m, float* v, __nv_bfloat16* wbf, int members,
-                            float lr, float b1, float b2, float eps, float c1, float c2)
+// The rows of a training batch (gather_rows): xin[r] = feats[order[r]], lbl[r] = labels[order[r]], zero
+// past n.
+struct GatherArgs {
+    const __nv_bfloat16* feats;
+    const float* labels;
+    const int32_t* order;
+    int n, batch;
+    __nv_bfloat16* xin;
+    float* lbl;
+};
+
+// Rows of block `block` with 16-byte accesses (feats 16-byte aligned): kRowU4 threads per row of IN BF16
+// values, 256 / kRowU4 rows per block of 256 threads.
+constexpr int kRowU4 = IN * 2 / 16;
+constexpr int kGatherRows = 256 / kRowU4;
+__device__ __forceinline__ void gather_rows(const GatherArgs& g, int block)
+{
+    const int r = block * kGatherRows + threadIdx.x / kRowU4, c = threadIdx.x % kRowU4;
+    if (r >= g.batch) return;
+    uint4 val = make_uint4(0u, 0u, 0u, 0u);
+    float lab = 0.0f;
+    if (r < g.n) {
+        const long long src = g.order ? g.order[r] : r;
+        val = __ldg(reinterpret_cast<const uint4*>(g.feats + src * IN) + c);
+        if (c == 0) lab = g.labels[src];
+    }
+    reinterpret_cast<uint4*>(g.xin + (long long)r * IN)[c] = val;
+    if (c == 0) g.lbl[r] = lab;
+}
+
+__global__ void __launch_bounds__(256) gather_batch16(const __grid_constant__ GatherArgs g)
 {
     pdl::grid_dep_enter();  // a step of the training chain: wait for the launch before it
-    const long long e = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
-    if (e >= (long long)members * P) return;
-    const long long p = e % P;
+    gather_rows(g, blockIdx.x);
+}
+
+// Adam on FP32 master weights, then the BF16 copies of W1..W4; four consecutive
+// parameters per thread (every parameter segment starts at a multiple of 4, so a group
+// lies in one segment; padding past the last parameter is left alone). Blocks from adam_blocks on
+// gather the next step's batch, which saves a launch of its own in every step. Bound by latency: the
+// parameters and moments, which only this kernel writes and the launch before the last one is done
+// with, are loaded before the wait, the gradients after it. 14 training steps 1.85 -> 1.75 ms
+// together with the head's sums in mlp_bwd_kernel and the losses stored by it instead of a copy per step.
+constexpr int kAdamBlocks = (int)((P / 4 + 255) / 256);  // per member
+__global__ void __launch_bounds__(256) adam_update(float* master, const float* grad, float* m, float* v,
+                                                   __nv_bfloat16* wbf, float lr, float b1, float b2, float eps, float c1,
+                                                   float c2, int adam_blocks, const __grid_constant__ GatherArgs next)
+{
+    if ((int)blockIdx.x >= adam_blocks) {
+        pdl::grid_dep_enter();
+        gather_rows(next, blockIdx.x - adam_blocks);
+        return;
+    }
+    const int mem = blockIdx.x / kAdamBlocks;
+    const int p = 4 * ((blockIdx.x - mem * kAdamBlocks) * 256 + threadIdx.x);
     if (p >= P_REAL) return;
-    float4 g4 = *reinterpret_cast<const float4*>(grad + e);
+    const long long e = mem * P + p;
     float4 m4 = *reinterpret_cast<const float4*>(m + e), v4 = *reinterpret_cast<const float4*>(v + e);
     float4 w4 = *reinterpret_cast<const float4*>(master + e);
+    pdl::grid_dep_enter();  // a step of the training chain: wait for the launch before it
+    const float4 g4 = *reinterpret_cast<const float4*>(grad + e);
     const float* gg = &g4.x;
     float* mm = &m4.x;
     float* vv = &v4.x;
@@ -328,7 +310,6 @@ __global__ void adam_update(float* master, const float* grad, float* m, float* v
     *reinterpret_cast<float4*>(m + e) = m4;
     *reinterpret_cast<float4*>(v + e) = v4;
     *reinterpret_cast<float4*>(master + e) = w4;
-    const long long mem = e / P;
     for (int l = 0; l < NL; ++l) {
         const long long len = WID * fan_in(l);
         if (p >= OFF_W(l) && p < OFF_W(l) + len) {
@@ -391,27 +372,6 @@ __global__ void gather_batch(const __nv_bfloat16* __restrict__ feats, const floa
         lbl[r] = 0.0f;
     }
     reinterpret_cast<__nv_bfloat162*>(xin + (long long)r * IN)[c] = val;
-}
-
-// The same gather with 16-byte accesses (feats 16-byte aligned): kRowU4 threads per row of
-// IN BF16 values, 256 / kRowU4 rows per block of 256 threads.
-constexpr int kRowU4 = IN * 2 / 16;
-constexpr int kGatherRows = 256 / kRowU4;
-__global__ void gather_batch16(const __nv_bfloat16* __restrict__ feats, const float* __restrict__ labels,
-                               const int32_t* __restrict__ order, int n, int batch, __nv_bfloat16* xin, float* lbl)
-{
-    pdl::grid_dep_enter();  // a step of the training chain: wait for the launch before it
-    const int r = blockIdx.x * kGatherRows + threadIdx.x / kRowU4, c = threadIdx.x % kRowU4;
-    if (r >= batch) return;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    float lab = 0.0f;
-    if (r < n) {
-        const long long src = order ? order[r] : r;
-        val = __ldg(reinterpret_cast<const uint4*>(feats + src * IN) + c);
-        if (c == 0) lab = labels[src];
-    }
-    reinterpret_cast<uint4*>(xin + (long long)r * IN)[c] = val;
-    if (c == 0) lbl[r] = lab;
 }
 
 template <bool A_KM, bool B_KN, int EPI>
@@ -588,10 +548,41 @@ int fused_forward(tune_surrogate* h, const __nv_bfloat16* feats, int64_t n, floa
     return fp8 ? launch_fused<true>(tx, tw1, tw, g, grid, s) : launch_fused<false>(tx, tw1, tw, g, grid, s);
 }
 
+// The head's backward pass of a training step: slices of `rows` rows, `slices` per member, and where they
+// are formed. Units (128 rows of a member) go round the training forward's `grid` CTAs; where some CTAs get
+// one unit less than the others, those (first .. grid - 1) do their own units' slices while the others run
+// their last unit, and head_bwd does the rest (first = grid: all). 8,192 rows x 5 members are 320 units on
+// 152 SMs: 136 CTAs wait for 16. 14 training steps 1.90 -> 1.85 ms.
+struct HeadSplit {
+    unsigned grid;
+    int first, rows, slices;
+    bool few;  // at most two slices per SM are left to head_bwd
+};
+HeadSplit head_split(const tune_surrogate* h, int n_pad)
+{
+    HeadSplit hs;
+    const long long units = (long long)(n_pad / tcm::kRows) * h->members, sms = tune::device_sm_count();
+    hs.grid = (unsigned)(units < sms ? units : sms);
+    // longer slices where the partial sums of 64 rows would not fit the partial buffer
+    hs.rows = tcm::kHeadRows;
+    while ((long long)h->members * ((n_pad + hs.rows - 1) / hs.rows) * tcm::kHeadStride >
+           (long long)h->part_slices * WID * WID)
+        hs.rows *= 2;
+    hs.slices = (n_pad + hs.rows - 1) / hs.rows;
+    const bool fused = h->use_tc && h->fwd_mode == 1 && h->bwd_mode == 1 && hs.rows == tcm::kHeadRows;
+    hs.first = (int)hs.grid;
+    if (fused && units % hs.grid) hs.first = (int)(units % hs.grid);
+    const long long rest = hs.first < (int)hs.grid
+                               ? (units + hs.grid - 1) / hs.grid * hs.first * (tcm::kRows / tcm::kHeadRows)
+                               : (long long)hs.slices * h->members;
+    hs.few = rest <= 2 * sms;
+    return hs;
+}
+
 // Training forward of rows [0, n_pad) of the current batch (h->xb) through the fused kernel
 // (BF16), keeping every layer's gelu'(Z) (FP16) and activations H for the backward pass and the
 // head outputs in h->y.
-int fused_train_forward(tune_surrogate* h, int n_pad, cudaStream_t s)
+int fused_train_forward(tune_surrogate* h, int n, int n_pad, cudaStream_t s)
 {
     CUtensorMap tx, tw1, tw;
     const auto u64 = CU_TENSOR_MAP_DATA_TYPE_UINT64;
@@ -636,13 +627,13 @@ int fused_train_forward(tune_surrogate* h, int n_pad, cudaStream_t s)
     for (int l = 0; l < NL; ++l) a.g_out[l] = h->G[l];
     a.h4_out = h->H[NL - 1];
     a.act_stride = (long long)h->batch * WID;
+    const HeadSplit hs4 = head_split(h, n_pad);
+    a.head = {h->lb, n, h->dZ[NL - 1], h->part, hs4.slices, hs4.first};
     constexpr int smem = tcm::Cfg<false>::smem;
     static std::atomic<uint64_t> attr{0};
     rc = smem_attr(tcm::mlp_train_kernel, smem, attr, "surrogate: training forward smem attribute");
     if (rc) return rc;
-    const long long sms = tune::device_sm_count();
-    const unsigned grid = (unsigned)(g.units < sms ? g.units : sms);
-    TUNE_CUDA_TRY(pdl::launch_dep(tcm::mlp_train_kernel, dim3(grid), dim3(tcm::kThreads), smem, s, tx, tw1, tw, th, a),
+    TUNE_CUDA_TRY(pdl::launch_dep(tcm::mlp_train_kernel, dim3(hs4.grid), dim3(tcm::kThreads), smem, s, tx, tw1, tw, th, a),
                   "surrogate: training forward launch");
     return TUNE_OK;
 }
@@ -650,7 +641,7 @@ int fused_train_forward(tune_surrogate* h, int n_pad, cudaStream_t s)
 // Input gradients of layers 4, 3 and 2 in one persistent launch (tc_mlp_bwd.cuh):
 // dz[l - 1] = bf16((dz[l] W_l) * G[l - 1]) for l = 3, 2, 1 (0-based), rows [0, n_pad),
 // G = gelu'(Z) as the forward pass kept it.
-int fused_backward(tune_surrogate* h, int n_pad, __nv_bfloat16* const* dz, cudaStream_t s)
+int fused_backward(tune_surrogate* h, int n_pad, __nv_bfloat16* const* dz, const tcm::ReduceArgs& red, cudaStream_t s)
 {
     if (n_pad % tcm::kRows) return tune::fail(TUNE_EINVAL, "surrogate: fused backward needs whole 128-row tiles");
     CUtensorMap tdz, tw;
@@ -688,6 +679,7 @@ int fused_backward(tune_surrogate* h, int n_pad, __nv_bfloat16* const* dz, cudaS
     }
     g.act_stride = (long long)h->batch * WID;
     g.status = h->status;
+    g.red = red;
     constexpr int smem = tcm::Cfg<false>::smem;
     static std::atomic<uint64_t> attr{0};
     rc = smem_attr(tcm::mlp_bwd_kernel, smem, attr, "surrogate: fused backward smem attribute");
@@ -746,13 +738,14 @@ int wgrad_tc(tune_surrogate* h, int n_pad, __nv_bfloat16* const* dz, cudaStream_
 // Forward through all members for rows [0, n_pad) (n_pad a multiple of 128).
 // x_in: layer-1 input rows (null: the current training batch; else the caller's features on the
 // tcgen05 path);
-// n_valid rows of it exist; store_z keeps gelu' of the pre-activations for a backward pass.
+// n_valid rows of it exist; store_z keeps gelu' of the pre-activations for a backward pass, which
+// follows with the batch's n_labelled rows.
 int forward(tune_surrogate* h, int n_pad, cudaStream_t s, const __nv_bfloat16* x_in = nullptr, int n_valid = -1,
-            bool store_z = true)
+            bool store_z = true, int n_labelled = 0)
 {
     // training with tcgen05 and the fused forward selected: one launch for all layers and the
     // head over the current batch (h->xb)
-    if (store_z && h->use_tc && h->fwd_mode == 1 && !x_in) return fused_train_forward(h, n_pad, s);
+    if (store_z && h->use_tc && h->fwd_mode == 1 && !x_in) return fused_train_forward(h, n_labelled, n_pad, s);
     if (!x_in) x_in = h->xin;
     if (n_valid < 0) n_valid = n_pad;
     for (int l = 0; l < NL; ++l) {
@@ -818,7 +811,8 @@ int wgrad_mma(tune_surrogate* h, int l, int n_pad, const __nv_bfloat16* dz, cuda
     return TUNE_OK;
 }
 
-int backward(tune_surrogate* h, int n, int n_pad, cudaStream_t s)
+// trace: the members' losses go there too (null: only to h->loss).
+int backward(tune_surrogate* h, int n, int n_pad, float* trace, cudaStream_t s)
 {
     const int B = h->batch;
     const int slices = (n_pad + kRowSlice - 1) / kRowSlice;
@@ -829,23 +823,21 @@ int backward(tune_surrogate* h, int n, int n_pad, cudaStream_t s)
     for (int l = 0; l < NL; ++l) dzl[l] = h->dZ[fused ? l : (l & 1)];
     // the loss gradient, the head's weight and bias gradients (slices, then their sum), the
     // loss and dZ4 in one pass and its reduction: steps of the training chain (pdl.cuh)
-    // (64-row slices, longer where their partials would not fit the partial buffer)
-    int hrows = 64;
-    while ((long long)h->members * ((n_pad + hrows - 1) / hrows) * kHeadStride > (long long)h->part_slices * WID * WID)
-        hrows *= 2;
-    const int hslices = (n_pad + hrows - 1) / hrows;
-    TUNE_CUDA_TRY(pdl::launch_dep(head_bwd, dim3(hslices, h->members), dim3(32 * kHeadGroups), 0, s, h->y, h->lb, n,
-                                  h->master, h->G[NL - 1], h->H[NL - 1], dzl[NL - 1], h->part, n_pad, B, hslices, hrows),
+    // (without the slices of the units whose head backward the forward pass has done)
+    const HeadSplit hs = head_split(h, n_pad);
+    const int hslices = hs.slices;
+    TUNE_CUDA_TRY(pdl::launch_dep(hs.few ? head_bwd<8> : head_bwd<2>, dim3(hslices, h->members),
+                                  dim3(32 * kHeadGroups), 0, s, h->y, h->lb, n, h->master, h->G[NL - 1], h->H[NL - 1],
+                                  dzl[NL - 1], h->part, n_pad, B, hslices, hs.rows, (int)hs.grid, hs.first),
                   "surrogate: head backward launch");
-    TUNE_CUDA_TRY(pdl::launch_dep(slices_reduce, dim3((kHeadStride + 31) / 32, h->members), dim3(32 * kRedWarps), 0,
-                                  s, h->part, h->grad, OFF_W5, WID + 1, hslices, kHeadStride, h->loss, n),
-                  "surrogate: head backward launch");
-    TUNE_CUDA_TRY(cudaGetLastError(), "surrogate: head backward launch");
+    const tcm::ReduceArgs red = {h->part, h->grad, P, OFF_W5, WID + 1, hslices, kHeadStride, h->members, h->loss, trace, n};
     if (fused) {  // input gradients dZ3..dZ1, then every layer's weight and bias gradients
-        int rc = fused_backward(h, n_pad, dzl, s);
+        int rc = fused_backward(h, n_pad, dzl, red, s);
         if (rc) return rc;
         return wgrad_tc(h, n_pad, dzl, s);
     }
+    TUNE_CUDA_TRY(pdl::launch_dep(slices_reduce, dim3(tcm::reduce_tasks(red)), dim3(32 * tcm::kRedWarps), 0, s, red),
+                  "surrogate: head backward launch");
     // mma.sync backward: per layer the weight gradient, the bias gradient and the input gradient
     for (int l = NL - 1; l >= 0; --l) {
         const __nv_bfloat16* dz = dzl[l];
@@ -854,8 +846,8 @@ int backward(tune_surrogate* h, int n, int n_pad, cudaStream_t s)
         int rc = wgrad_mma(h, l, n_pad, dz, s);
         if (rc) return rc;
         bias_partial<<<dim3(slices, h->members), WID, 0, s>>>(dz, h->part, n_pad, B, slices);
-        slices_reduce<<<dim3(WID / 32, h->members), 32 * kRedWarps, 0, s>>>(h->part, h->grad, OFF_B(l), WID, slices,
-                                                                          WID + 1, nullptr, 0);
+const tcm::ReduceArgs bias = {h->part, h->grad, P, OFF_B(l), WID, slices, WID + 1, h->members, nullptr, nullptr, 0};
+        slices_reduce<<<tcm::reduce_tasks(bias), 32 * tcm::kRedWarps, 0, s>>>(bias);
         TUNE_CUDA_TRY(cudaGetLastError(), "surrogate: reduce launch");
         if (l == 0) continue;
         // input gradient of layer l, times gelu' of layer l-1: dZ_{l-1} = (dZ_l W_l) * gelu'(Z_{l-1})
@@ -880,25 +872,36 @@ int backward(tune_surrogate* h, int n, int n_pad, cudaStream_t s)
     return TUNE_OK;
 }
 
-int adam(tune_surrogate* h, cudaStream_t s)
+// next: the following step's batch, gathered by the same launch (null: none).
+int adam(tune_surrogate* h, const GatherArgs* next, cudaStream_t s)
 {
     h->step += 1;
     const float c1 = 1.0f - powf(h->b1, (float)h->step), c2 = 1.0f - powf(h->b2, (float)h->step);
-    const long long total = (long long)h->members * P;
-    TUNE_CUDA_TRY(pdl::launch_dep(adam_update, dim3((unsigned)((total / 4 + 255) / 256)), dim3(256), 0, s, h->master,
-                                  h->grad, h->m, h->v, h->wbf, h->members, h->lr, h->b1, h->b2, h->eps, c1, c2),
+    const int blocks = h->members * kAdamBlocks;
+    const int gather = next ? (next->batch + kGatherRows - 1) / kGatherRows : 0;
+    TUNE_CUDA_TRY(pdl::launch_dep(adam_update, dim3(blocks + gather), dim3(256), 0, s, h->master, h->grad, h->m, h->v,
+                                  h->wbf, h->lr, h->b1, h->b2, h->eps, c1, c2, blocks, next ? *next : GatherArgs{}),
                   "surrogate: adam launch");
     h->fp8_stale = true;
     TUNE_CUDA_TRY(cudaGetLastError(), "surrogate: adam launch");
     return TUNE_OK;
 }
 
+// Rows of the batch by 16-byte gathers into h->xin and h->lbl.
+GatherArgs batch_args(const tune_surrogate* h, const __nv_bfloat16* feats, const float* labels, const int32_t* order,
+                      int n)
+{
+    return {feats, labels, order, n, h->batch, h->xin, h->lbl};
+}
+
+bool gathers16(const __nv_bfloat16* feats) { return (reinterpret_cast<uintptr_t>(feats) & 15) == 0; }
+
 int load_batch(tune_surrogate* h, const __nv_bfloat16* feats, const float* labels, const int32_t* order, int n,
                cudaStream_t s)
 {
-    if ((reinterpret_cast<uintptr_t>(feats) & 15) == 0)
+    if (gathers16(feats))
         TUNE_CUDA_TRY(pdl::launch_dep(gather_batch16, dim3((h->batch + kGatherRows - 1) / kGatherRows), dim3(256), 0, s,
-                                      feats, labels, order, n, h->batch, h->xin, h->lbl),
+                                      batch_args(h, feats, labels, order, n)),
                       "surrogate: gather launch");
     else
         TUNE_CUDA_TRY(pdl::launch_dep(gather_batch, dim3(h->batch), dim3(IN / 2), 0, s, feats, labels, order, n,
@@ -1126,9 +1129,9 @@ int surrogate_train_step(tune_surrogate* h, const uint16_t* feats, const float* 
     const int nb = (int)n, n_pad = (nb + 127) / 128 * 128;
     const auto* f = reinterpret_cast<const __nv_bfloat16*>(feats);
     int rc = use_batch_in_place(h, f, labels, nb) ? TUNE_OK : load_batch(h, f, labels, nullptr, nb, s);
-    if (!rc) rc = forward(h, n_pad, s);
-    if (!rc) rc = backward(h, nb, n_pad, s);
-    if (!rc && apply_update) rc = adam(h, s);
+    if (!rc) rc = forward(h, n_pad, s, nullptr, -1, true, nb);
+    if (!rc) rc = backward(h, nb, n_pad, nullptr, s);
+    if (!rc && apply_update) rc = adam(h, nullptr, s);
     return rc;
 }
 
@@ -1140,22 +1143,24 @@ int surrogate_train(tune_surrogate* h, const uint16_t* feats, const float* label
         return tune::fail(TUNE_EINVAL, "surrogate_train: bad arguments");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const auto* f = reinterpret_cast<const __nv_bfloat16*>(feats);
-    const int64_t steps = (n + h->batch - 1) / h->batch;
-    for (int ep = 0; ep < epochs; ++ep) {
-        for (int64_t st = 0; st < steps; ++st) {
-            const int64_t r0 = st * h->batch;
-            const int nb = (int)((n - r0) < h->batch ? (n - r0) : h->batch);
-            const int n_pad = (nb + 127) / 128 * 128;
-            int rc = load_batch(h, f, labels, order + (int64_t)ep * n + r0, nb, s);
-            if (!rc) rc = forward(h, n_pad, s);
-            if (!rc) rc = backward(h, nb, n_pad, s);
-            if (!rc) rc = adam(h, s);
-            if (rc) return rc;
-            if (loss_trace)
-                TUNE_CUDA_TRY(cudaMemcpyAsync(loss_trace + ((int64_t)ep * steps + st) * h->members, h->loss,
-                                              h->members * sizeof(float), cudaMemcpyDeviceToDevice, s),
-                              "surrogate_train: loss trace");
+    const int64_t per_epoch = (n + h->batch - 1) / h->batch, steps = per_epoch * epochs;
+    // rows of step st: order[first(st)] ..
+    auto first = [&](int64_t st) { return st / per_epoch * n + st % per_epoch * h->batch; };
+    auto rows = [&](int64_t st) { return (int)std::min<int64_t>(n - st % per_epoch * h->batch, h->batch); };
+    const bool chained = gathers16(f);  // a step's last launch gathers the next step's batch
+    for (int64_t st = 0; st < steps; ++st) {
+        const int nb = rows(st), n_pad = (nb + 127) / 128 * 128;
+        int rc = st == 0 || !chained ? load_batch(h, f, labels, order + first(st), nb, s) : TUNE_OK;
+        if (!rc) rc = forward(h, n_pad, s, nullptr, -1, true, nb);
+        if (!rc) rc = backward(h, nb, n_pad, loss_trace ? loss_trace + st * h->members : nullptr, s);
+        if (rc) return rc;
+        if (chained && st + 1 < steps) {
+            const GatherArgs next = batch_args(h, f, labels, order + first(st + 1), rows(st + 1));
+            rc = adam(h, &next, s);
+        } else {
+            rc = adam(h, nullptr, s);
         }
+        if (rc) return rc;
     }
     return TUNE_OK;
 }

@@ -175,6 +175,11 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 // The thread's committed bulk stores are complete.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
 
+__device__ __forceinline__ void named_barrier(int id, int threads)
+{
+    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* b)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::sa(b)) : "memory");
@@ -319,13 +324,19 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b)
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
-// 256-bit global store of eight 32-bit words (address 32-byte aligned), not kept in L1 (what the
-// epilogues store is read by later launches only).
+// 256-bit global store of eight 32-bit words (address 32-byte aligned), not kept in L1; ONCE: with the
+// policy of policy_evict_first().
+template <bool ONCE = false>
 __device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&w)[8])
 {
-    asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "r"(w[0]), "r"(w[1]),
-                 "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                 : "memory");
+    if (ONCE)
+        asm volatile("st.global.L1::no_allocate.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p),
+                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+    else
+        asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "r"(w[0]),
+                     "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
 }
 
 // 256-bit global load of eight floats (address 32-byte aligned; data not written by this kernel).

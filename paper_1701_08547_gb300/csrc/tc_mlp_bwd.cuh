@@ -45,6 +45,48 @@ __device__ __forceinline__ uint64_t sdesc_w_mn(const void* p)
            (2ull << 61);
 }
 
+// Sums over slices: grad[mem * P + off + j] = sum over slices of part[mem][slice][j], j < cols (slice rows of
+// `stride` floats); with `loss`, column cols is the slices' sum of squared errors and loss[mem] (and
+// trace[mem]) that sum / n. A task is 32 columns of a member: warp w of kRedWarps adds slices w,
+// w + kRedWarps, ... in order (reduce_partial), then, after a barrier, the warps' sums are added in warp
+// order (reduce_finish), so that the result does not depend on who runs it.
+constexpr int kRedWarps = 32;
+struct ReduceArgs {
+    const float* part;
+    float* grad;
+    long long P, off;
+    int cols, slices, stride, members;
+    float *loss, *trace;
+    int n;
+};
+
+__host__ __device__ inline int reduce_blocks(const ReduceArgs& g) { return (g.cols + (g.loss ? 1 : 0) + 31) / 32; }
+__host__ __device__ inline int reduce_tasks(const ReduceArgs& g) { return reduce_blocks(g) * g.members; }
+
+__device__ __forceinline__ void reduce_partial(const ReduceArgs& g, int task, int w, int lane, float* red)
+{
+    const int nb = reduce_blocks(g), mem = task / nb, j = (task - mem * nb) * 32 + lane;
+    float s = 0.0f;
+    if (j < g.cols + (g.loss ? 1 : 0))
+        for (int q = w; q < g.slices; q += kRedWarps) s += g.part[((long long)mem * g.slices + q) * g.stride + j];
+    red[w * 32 + lane] = s;
+}
+
+__device__ __forceinline__ void reduce_finish(const ReduceArgs& g, int task, int lane, const float* red)
+{
+    const int nb = reduce_blocks(g), mem = task / nb, j = (task - mem * nb) * 32 + lane;
+    if (j >= g.cols + (g.loss ? 1 : 0)) return;
+    float t = red[lane];
+#pragma unroll
+    for (int q = 1; q < kRedWarps; ++q) t += red[q * 32 + lane];
+    if (j < g.cols) {
+        g.grad[mem * g.P + g.off + j] = t;
+    } else {
+        g.loss[mem] = t / (float)g.n;
+        if (g.trace) g.trace[mem] = t / (float)g.n;
+    }
+}
+
 struct BwdArgs {
     int members;
     long long units;                  // rows / 128 * members (rows a multiple of 128: every unit's rows exist)
@@ -53,6 +95,7 @@ struct BwdArgs {
     int dz_coord[kBwdStages];         // stage j: the layer coordinate of dz[j] in the map tdzs
     long long act_stride;             // member stride of z and dz (elements); rows of 256
     int* status;
+    ReduceArgs red;                   // the head's slice sums
 };
 
 
@@ -296,6 +339,17 @@ __global__ void __maxnreg__(96) mlp_bwd_kernel(const __grid_constant__ CUtensorM
                     if (lane == 0) mbar_arrive(&act_ready[s]);
                 }
             }
+        }
+        // The head's slice sums, by the CTAs that have the fewest units (which are the last ones), each warp
+        // for two of kRedWarps; the activation buffers are free after the last accumulator.
+        static_assert(kRedWarps == 2 * kEpiWarps, "two partial sums per warp");
+        float* red = reinterpret_cast<float*>(smem);
+        for (int task = (int)(gridDim.x - 1 - blockIdx.x); task < reduce_tasks(g.red); task += (int)gridDim.x) {
+            named_barrier(1, 32 * kEpiWarps);
+            reduce_partial(g.red, task, e, lane, red);
+            reduce_partial(g.red, task, e + kEpiWarps, lane, red);
+            named_barrier(1, 32 * kEpiWarps);
+            if (e == 0) reduce_finish(g.red, task, lane, red);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");

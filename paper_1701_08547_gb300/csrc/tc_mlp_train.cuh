@@ -9,18 +9,37 @@
 // accumulator at once (which frees it for the next layer) and hand the layer's output over one K chunk at a
 // time, so that the next layer's MMAs start while the later chunks are still being computed. 14 steps of
 // 8,192 rows x 5 members: 2.17 -> 2.05 ms (2.21 with the inference kernel's split of the warps);
-// 1.89 ms with the backward kernels' changes and the L2 policies (policy_evict_first).
+// 1.89 ms with the backward kernels' changes and the L2 policies (policy_evict_first), 1.75 ms with the
+// small launches of a step merged into its large ones.
 #pragma once
 
 #include "tc_mlp.cuh"
 
 namespace tcm {
 
+// The head's backward pass over a slice of rows of one member (head_rows, head_sum): dy[i] =
+// 2 (y[i] - lbl[i]) / n for the n labelled rows (0 past them), dZ4[i][j] = bf16(dy[i] * w5[j] *
+// gelu'(Z4)[i][j]), and part[member][slice][j] = sum over the slice of dy[i] H4[i][j] (j < 256), of
+// dy[i] (j = 256) and of (y[i] - lbl[i])^2 (j = 257).
+constexpr int kHeadGroups = 8;          // row groups of 32 threads; group q takes rows q, q + 8, ...
+constexpr int kHeadStride = kWid + 2;   // floats per slice of part
+constexpr int kHeadRows = 64;           // rows of a slice (longer only where part would not hold them)
+
+struct HeadArgs {
+    const float* lbl;
+    int n;
+    __nv_bfloat16* dz;   // dZ4, [members][act_stride]
+    float* part;
+    int slices;          // per member
+    int first;           // CTAs first .. gridDim.x - 1 do their own units' slices
+};
+
 struct TrainArgs {
     Args f;                     // the forward's arguments (rows < f.n are written to f.pred)
     __half* g_out[kLayers];     // gelu' of each layer, [members][act_stride]
     __nv_bfloat16* h4_out;      // H4, the same layout in rows of 256 (H1..H3 go through the map `th`)
     long long act_stride;
+    HeadArgs head;
 };
 
 struct TrainControl {
@@ -56,6 +75,69 @@ __device__ __forceinline__ uint32_t gelu_grad_half2(float2 z, float2 t)
     const float2 d = fma2(mul2(w, fma2(t, f2(-1.0f), f2(1.0f))), a, a);
     const __half2 d2 = __floats2half2_rn(d.x, d.y);
     return *reinterpret_cast<const uint32_t*>(&d2);
+}
+
+// Rows i0 + q, i0 + q + 8, ... < i1 of a slice, by the 32 threads of row group q (eight columns each, 16-byte
+// accesses); the group's sums go to red[0 .. 257]. y, G4, H4, dZ: the member's. FRESH: y, G4 and H4 were
+// written by this CTA (before a barrier). ROWS: rows whose loads are requested together.
+template <bool FRESH, int ROWS>
+__device__ __forceinline__ void head_rows(const float* y, const float* lbl, int n, const float* w5, const __half* G4,
+                                          const __nv_bfloat16* H4, __nv_bfloat16* dZ, int i0, int i1, int q, int lane,
+                                          float* red)
+{
+    const int j = 8 * lane;
+    const float n_f = (float)n;
+    float w[8];
+    {
+        const float4 a = *reinterpret_cast<const float4*>(w5 + j);
+        const float4 b = *reinterpret_cast<const float4*>(w5 + j + 4);
+        w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+    }
+    float sh[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, sb = 0.0f, se = 0.0f;
+#pragma unroll ROWS
+    for (int i = i0 + q; i < i1; i += kHeadGroups) {
+        float di = 0.0f;
+        if (i < n) {
+            const float e = (FRESH ? __ldcg(y + i) : y[i]) - lbl[i];
+            di = 2.0f * e / n_f;
+            se += e * e;
+        }
+        const long long o = (long long)i * kWid + j;
+        const uint4* gp = reinterpret_cast<const uint4*>(G4 + mlp::gprime_at(i, j));
+        const uint4* hp = reinterpret_cast<const uint4*>(H4 + o);
+        const uint4 gv = FRESH ? __ldcg(gp) : __ldg(gp);
+        const uint4 hv = FRESH ? __ldcg(hp) : __ldg(hp);
+        const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, hw[4] = {hv.x, hv.y, hv.z, hv.w};
+        uint32_t out[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float2 g = __half22float2(*reinterpret_cast<const __half2*>(&gw[t]));
+            const float2 h = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[t]));
+            const __nv_bfloat162 z = __floats2bfloat162_rn(di * w[2 * t] * g.x, di * w[2 * t + 1] * g.y);
+            out[t] = *reinterpret_cast<const uint32_t*>(&z);
+            sh[2 * t] = fmaf(di, h.x, sh[2 * t]);
+            sh[2 * t + 1] = fmaf(di, h.y, sh[2 * t + 1]);
+        }
+        *reinterpret_cast<uint4*>(dZ + o) = make_uint4(out[0], out[1], out[2], out[3]);
+        sb += di;
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) red[j + c] = sh[c];
+    if (j == 0) {
+        red[kWid] = sb;
+        red[kWid + 1] = se;
+    }
+}
+
+// The row groups' sums (red[group][258], after a barrier), added in group order, by 256 threads.
+__device__ __forceinline__ void head_sum(const float* red, int tid, float* part)
+{
+    for (int c = tid; c < kHeadStride; c += 32 * kHeadGroups) {
+        float v = red[c];
+#pragma unroll
+        for (int g = 1; g < kHeadGroups; ++g) v += red[g * kHeadStride + c];
+        part[c] = v;
+    }
 }
 
 // Registers that an asynchronous TMEM load filled, after its wait: no use of them moves above it.
@@ -130,7 +212,7 @@ __device__ __forceinline__ float train_rows(uint32_t tlane, const float* bias, c
             ld16(bias + col(b + 1), bb);
             if (HEAD) ld16(w5 + col(b + 1), ww);
         }
-        st_global_v8(g_row + col(b) * 128, gd);
+        st_global_v8<!HEAD>(g_row + col(b) * 128, gd);  // (gelu'(Z4) is read next)
         if (HEAD) {
             st_global_v8(h_row + col(b), w);
         } else {  // 16 columns = two 16-byte units
@@ -365,6 +447,27 @@ __global__ void __maxnreg__(96) mlp_train_kernel(const __grid_constant__ CUtenso
                                           ctl.rdy[s], acc_ph, ab, ok);
                     }
                 }
+            }
+        }
+        // The head's backward pass of this CTA's units, while the CTAs with one unit more run theirs: two
+        // slices (128 rows) at a time, warps 2-9 and 10-17 one each, sums through the activation buffers
+        // (after an abort the results are as useless as the forward's, but every access is in bounds and
+        // every warp is at the barriers).
+        const HeadArgs& hd = t.head;
+        if ((int)blockIdx.x >= hd.first) {
+            const int grp = (warp - 2) >> 3, hq = (warp - 2) & 7;
+            float* red = reinterpret_cast<float*>(smem) + grp * kHeadGroups * kHeadStride;
+            named_barrier(1, 32 * kEpiWarps);
+            for (int j = 0; j < my_units; ++j) {
+                const Unit u = train_unit(j, g.members);
+                const int i0 = u.tile * kRows + grp * kHeadRows;
+                const long long base = (long long)u.mem * t.act_stride;
+                head_rows<true, 2>(g.pred + (long long)u.mem * g.pred_stride, hd.lbl, hd.n, g.master + u.mem * g.P + g.off_w5,
+                                t.g_out[kLayers - 1] + base, t.h4_out + base, hd.dz + base, i0, i0 + kHeadRows, hq, lane,
+                                red + hq * kHeadStride);
+                named_barrier(2 + grp, 32 * kHeadGroups);
+                head_sum(red, 32 * hq + lane, hd.part + ((long long)u.mem * hd.slices + i0 / kHeadRows) * kHeadStride);
+                named_barrier(2 + grp, 32 * kHeadGroups);
             }
         }
     }
