@@ -19,9 +19,9 @@ __host__ __device__ __forceinline__ int ceil_div(int a, int b) { return (a + b -
 template <int M>
 __device__ __forceinline__ float neumaier(const float (&x)[M])
 {
-    float s = 0.0f, comp = 0.0f;
+    float s = x[0], comp = 0.0f;  // (0 + x[0] has no error)
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
+    for (int i = 1; i < M; ++i) {
         float t = __fadd_rn(s, x[i]);
         if (fabsf(s) >= fabsf(x[i]))
             comp = __fadd_rn(comp, __fadd_rn(__fsub_rn(s, t), x[i]));
@@ -120,15 +120,22 @@ constexpr float kMaxCount = 0x1p40f;
 // Malformed descriptor: mask outside the axes, or a field out of range (counts
 // outside [0, 2^40] or not a number, d outside [0, 1], r0 outside [0, 2^24),
 // s0 outside [0, 2^30)).
-__device__ __forceinline__ bool desc_bad(const Desc& k, const tune_axes& x)
+__device__ __forceinline__ bool count_bad(float n) { return !(n >= 0.0f && n <= kMaxCount); }
+
+// The same without the counts.
+__device__ __forceinline__ bool desc_fields_bad(const Desc& k, const tune_axes& x)
 {
     const uint32_t t_ok = x.n_t == 32 ? 0xffffffffu : ((1u << x.n_t) - 1u);
     const uint32_t g_ok = (1u << x.n_g) - 1u, u_ok = (1u << x.n_u) - 1u, c_ok = (1u << x.n_c) - 1u;
-    bool bad = k.top != 0 || (k.tm & ~t_ok) || (k.gm & ~g_ok) || (k.um & ~u_ok) || (k.cm & ~c_ok) ||
-               k.r0 < 0 || k.r0 >= (1 << 24) || k.s0 < 0 || k.s0 >= (1 << 30) ||
-               !(k.d >= 0.0f && k.d <= 1.0f);
+    return k.top != 0 || (k.tm & ~t_ok) || (k.gm & ~g_ok) || (k.um & ~u_ok) || (k.cm & ~c_ok) || k.r0 < 0 ||
+           k.r0 >= (1 << 24) || k.s0 < 0 || k.s0 >= (1 << 30) || !(k.d >= 0.0f && k.d <= 1.0f);
+}
+
+__device__ __forceinline__ bool desc_bad(const Desc& k, const tune_axes& x)
+{
+    bool bad = desc_fields_bad(k, x);
 #pragma unroll
-    for (int c = 0; c < 7; ++c) bad = bad || !(k.n[c] >= 0.0f && k.n[c] <= kMaxCount);
+    for (int c = 0; c < 7; ++c) bad = bad || count_bad(k.n[c]);
     return bad;
 }
 

@@ -43,7 +43,7 @@ void host_cta_tables(const tune_arch& a, const tune_axes& x, CtaTables& ct)
         float mn = inf;
         for (int g = 0; g < x.n_g; ++g) mn = std::min(mn, ct.ipar[b][g]);
         ct.iparmin[b] = mn;
-        unsigned char* ord = ct.perm[b];
+        unsigned char ord[16] = {};
         for (int g = 0; g < x.n_g; ++g) {
             const float v = ct.ipar[b][g];
             int j = g;
@@ -52,6 +52,10 @@ void host_cta_tables(const tune_arch& a, const tune_axes& x, CtaTables& ct)
                 --j;
             }
             ord[j] = (unsigned char)g;
+        }
+        for (int r = 0; r < x.n_g; ++r) {
+            ct.rperm[b][15 - r] = ord[r];
+            ct.place[b] |= (unsigned long long)(15 - r) << (4 * ord[r]);
         }
         for (int r = 0; r + 1 < x.n_g; ++r) {
             const float v1 = ct.ipar[b][ord[r]], v2 = ct.ipar[b][ord[r + 1]];
@@ -84,8 +88,9 @@ void host_cta_tables(const tune_arch& a, const tune_axes& x, CtaTables& ct)
     for (int R = 0; R < 256; ++R) {
         int warps, wbmax;
         reg_params(a, R, warps, wbmax);
-        ct.rwarps[R] = (unsigned short)warps;
-        ct.rwbmax[R] = (unsigned short)std::min(wbmax, 65535);
+        ct.rwarps[R] = (unsigned char)warps;
+        // (a block of more than kMaxW warps has G_W = 0, so the limit beyond 255 does not matter)
+        ct.rwbmax[R] = (unsigned char)std::min(wbmax, 255);
     }
 }
 

@@ -22,10 +22,14 @@ struct CtaTables {
     int wb[32];                      // W_B = ceil(T / 32) by t position
     int gw[32];                      // G_W by t position (0 if T > max threads per block)
     unsigned char divt[kMaxW + 1][32];  // floor(w / W_B) by (w, t position)
-    unsigned char perm[kMaxB][16];   // g positions of ipar row b in increasing (value, g) order
+    // g positions of ipar row b in increasing (value, g) order, backwards: the first is [15], so that the
+    // highest set bit of a mask over these places is the next grid size; and the place of every g position,
+    // four bits each
+    unsigned char rperm[kMaxB][16];
+    unsigned long long place[kMaxB];
     float iparmin[kMaxB];            // min of ipar row b over all axis grid sizes
-    unsigned short rwarps[256];      // register-limited warps by R (Eq. 4, per-warp allocation)
-    unsigned short rwbmax[256];      // largest W_B whose block fits the per-block register limit, by R
+    unsigned char rwarps[256];       // register-limited warps by R (Eq. 4, per-warp allocation; at most kMaxW)
+    unsigned char rwbmax[256];       // largest W_B whose block fits the per-block register limit, by R, up to 255
     int cap_lo[4];                   // first capacity index allowed by carveout position c
     int order_safe;                  // 1: distinct ipar values of a row differ by more than 2^-21 relative
     int unit_shift;                  // log2 of the shared-memory allocation unit, or -1

@@ -24,6 +24,13 @@
 //    holds the j-th best); ties go to the lower canonical index.
 //  * with TUNE_EMIT_POINTS every point's B*, W* and cost is written after that, in
 //    canonical order.
+//
+// Bound by issue slots (about 80 % used). 100,000 dense kernels, k = 10: 216 -> 196 us; 1,000,000
+// uneven ones, k = 5: 1,434 -> 1,238 us; 317,078 of 128 points, k = 15: 1,267 -> 672 us, from walks over
+// the kernel's grid sizes by a mask of places instead of a scan of the row (1,361 us uneven), the
+// list of a batch left in shared memory until it is complete, candidates kept in triple order (so that
+// equal costs come in lane order and leave together), equal bounds counted together, two carveouts per
+// packed FP32 operation, and the descriptor and the unroll tables read as 16-byte words.
 #include <math.h>
 #include <stdint.h>
 
@@ -67,19 +74,20 @@ constexpr int kEmitAlone = 2048;
 
 
 struct WarpTables {
-    float iparmin[kMaxB + 1];  // by B*: min over the kernel's grid sizes of ipar(B*, G); [0] = NaN
+    alignas(8) float iparmin[kMaxB + 1];  // by B*: min over the kernel's grid sizes of ipar(B*, G); [0] = NaN
+    unsigned short places[kMaxB + 1];  // by B*: the kernel's grid sizes as places in rperm (not for a full set)
     unsigned char gwr[32][8];  // min(G_W, G_R) by (t rank, u rank)
-    float cnm[8], cm[8];     // by u rank
-    int regs[8];             // R by u rank
+    // by u rank: C_nm; C_m; register-limited warps | (largest W_B that fits) << 8; R (the last two as bits)
+    float4 uinfo[8];
     int gs[4];               // G_S by c rank
     int4 tinfo[32];          // by t rank: W_B, lane efficiency (float bits), t position, G_W
-    int ru[8];               // by u rank: register-limited warps | (largest W_B that fits) << 8
     int gpos[16];            // g position by g rank
     // emitting pass: the space's axis sizes (nT = 0: nothing to write), whether the (T, U) block limit is
     // formed in place, and the first point's place in the arrays
     int nT, nG, nU, nC, simple;
     int64_t off;
     union {
+        int4 desc[4];        // the descriptor's words, before the ranking pass
         float key[32 * 32];  // ranking pass: each triple's minimum cost, by (row, lane)
         struct {             // emitting pass, after the ranking:
             float iparc[kMaxB][kIparStride];  // ipar rows compacted to the kernel's grid sizes
@@ -99,6 +107,27 @@ __device__ __forceinline__ bool key_less(float c, int i, float c2, int i2)
     return c < c2 || (c == c2 && i < i2);
 }
 
+
+// Packed FP32 pairs (each result rounded to nearest as the scalar operation's).
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
+        " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mul.rn.f32x2 d, a, b;\n"
+        " mov.b64 {%0, %1}, d;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 
 template <int N>
 struct IntC {
@@ -136,12 +165,12 @@ __device__ __forceinline__ void warp_list_insert(float& lc, int& li, float& tau_
     tau_i = __shfl_sync(kFull, li, k - 1);
 }
 
-// min(G_W, G_R) of (t rank, u rank); ti = tinfo[t rank].
+// min(G_W, G_R) of (t rank, u rank); ti = tinfo[t rank], ui = uinfo[u rank].
 __device__ __forceinline__ int block_limit_of(const CtaTables& ct, const WarpTables& w, bool simple, int t_r, const int4& ti,
-                                              int u_r)
+                                              int u_r, const float4& ui)
 {
     if (!simple) return w.gwr[t_r][u_r];
-    const int ru = w.ru[u_r];
+    const int ru = __float_as_int(ui.z);
     return min(ti.w, ti.x > (ru >> 8) ? 0 : (int)ct.divt[ru & 0xff][ti.z]);
 }
 
@@ -161,12 +190,13 @@ __device__ __forceinline__ void emit_points(const CtaTables& ct, const WarpTable
         // of 32 consecutive points (a third of the instructions of the general walk)
         const int uc_r = lane & (nUC - 1), g0 = lane / nUC, dg = 32 / nUC;
         const int u_r = uc_r / nC, c = uc_r - u_r * nC;
-        const float cnm = w.cnm[u_r], cmv = w.cm[u_r];
+        const float4 ui = w.uinfo[u_r];
+        const float cnm = ui.x, cmv = ui.y;
         const int gs = w.gs[c];
         int64_t at = w.off + (int64_t)t_beg * g_stride + lane;
         for (int t_r = t_beg; t_r < t_end; ++t_r, at += g_stride) {
             const int4 ti = w.tinfo[t_r];
-            const int B = min(block_limit_of(ct, w, simple, t_r, ti, u_r), gs), W = B * ti.x;
+            const int B = min(block_limit_of(ct, w, simple, t_r, ti, u_r, ui), gs), W = B * ti.x;
             const float X = B > 0 ? __fmul_rn(__fmaf_rn(cmv, ct.hide[W], cnm), __int_as_float(ti.y)) : kInf;
             const float* row = w.iparc[max(B, 1) - 1];
             int64_t q = at;
@@ -196,8 +226,9 @@ __device__ __forceinline__ void emit_points(const CtaTables& ct, const WarpTable
             const int t_r = small_div(tri, rcp_uc), uc_r = tri - t_r * nUC;
             const int u_r = small_div(uc_r, rcp_c), c = uc_r - u_r * nC;
             const int4 ti = w.tinfo[t0 + t_r];
-            const int B = min(block_limit_of(ct, w, simple, t0 + t_r, ti, u_r), w.gs[c]), W = B * ti.x;
-            const float X = __fmul_rn(__fmaf_rn(w.cm[u_r], ct.hide[W], w.cnm[u_r]), __int_as_float(ti.y));
+            const float4 ui = w.uinfo[u_r];
+            const int B = min(block_limit_of(ct, w, simple, t0 + t_r, ti, u_r, ui), w.gs[c]), W = B * ti.x;
+            const float X = __fmul_rn(__fmaf_rn(ui.y, ct.hide[W], ui.x), __int_as_float(ti.y));
             tris[tri] = make_float2(B > 0 ? X : kInf, __int_as_float(B | (W << 8) | (((max(B, 1) - 1) * kIparStride) << 16)));
         }
         __syncwarp();
@@ -300,16 +331,16 @@ __global__ void __maxnreg__(64)
     };
     // ranks descriptor kid, whose four 16-byte words lanes 0..3 (mod 4) hold in v, on this warp
     auto rank = [&](const int64_t kid, const int4 v) {
-        int4 vw[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            vw[q] = make_int4(__shfl_sync(kFull, v.x, q), __shfl_sync(kFull, v.y, q),
-                              __shfl_sync(kFull, v.z, q), __shfl_sync(kFull, v.w, q));
+        if (lane < 4) w.desc[lane] = v;
+        __syncwarp();
+        const int4 vw[4] = {w.desc[0], w.desc[1], w.desc[2], w.desc[3]};
         Desc kd;
         unpack(vw, kd);
         const int r0 = kd.r0, s0 = kd.s0;
         const uint32_t tm = kd.tm, gm = kd.gm, um = kd.um, cm = kd.cm;
-        const bool bad = desc_bad(kd, x);
+        // (a count per lane: its words 0..6)
+        const bool bad = __any_sync(kFull, (lane < 7 && count_bad(reinterpret_cast<const float*>(w.desc)[lane])) ||
+                                               desc_fields_bad(kd, x));
         const int nT = __popc(tm), nG = __popc(gm), nU = __popc(um), nC = __popc(cm);
         if (bad || nT * nG * nU * nC == 0) {
             if (bad && lane == 0) atomicOr(status, tune::kStatusInvalid);
@@ -317,6 +348,7 @@ __global__ void __maxnreg__(64)
                 topk_idx[kid * k + lane] = -1;
                 topk_cost[kid * k + lane] = kInf;
             }
+            __syncwarp();  // the descriptor's words are rewritten
             return;
         }
         const int nUC = nU * nC;
@@ -330,8 +362,8 @@ __global__ void __maxnreg__(64)
             const int ur = __popc(um & below);
             const int U = x.u[lane];
             const int R = r0 + 4 * (U - 1);
-            unit_costs(kd.n, kd.d, U, ct.rcp, a.work_scale, w.cnm[ur], w.cm[ur]);
-            w.regs[ur] = R;
+            float cnm, cm_u;
+            unit_costs(kd.n, kd.d, U, ct.rcp, a.work_scale, cnm, cm_u);
             int warps, wbmax;
             if (R >= 0 && R < 256) {
                 warps = ct.rwarps[R];
@@ -339,7 +371,7 @@ __global__ void __maxnreg__(64)
             } else {
                 reg_params(a, R, warps, wbmax);
             }
-            w.ru[ur] = warps | (wbmax << 8);
+            w.uinfo[ur] = make_float4(cnm, cm_u, __int_as_float(warps | (wbmax << 8)), __int_as_float(R));
         }
         if (lane < 4 && ((cm >> lane) & 1u)) w.gs[__popc(cm & below)] = smem_blocks_from(a, ct, s0, lane);
         // Per-warp register allocation with R > 0 for every unroll (r0 > 0): the (T, U)
@@ -356,25 +388,31 @@ __global__ void __maxnreg__(64)
             w.tinfo[tr] = make_int4(wb, __float_as_int(ct.lane[lane]), lane, gw);
             if (!simple) {
                 for (int ur = 0; ur < nU; ++ur) {
-                    const int ru = w.ru[ur];
-                    const int gr = reg_blocks(a, ct, w.regs[ur], wb, lane, ru & 0xff, ru >> 8);
+                    const float4 ui = w.uinfo[ur];
+                    const int ru = __float_as_int(ui.z);
+                    const int gr = reg_blocks(a, ct, __float_as_int(ui.w), wb, lane, ru & 0xff, ru >> 8);
                     w.gwr[tr][ur] = (unsigned char)min(gw, gr);
                 }
             }
         }
-        auto block_limit = [&](int t_r, const int4& ti, int u_r) { return block_limit_of(ct, w, simple, t_r, ti, u_r); };
-        // ---- minima of the waves/slots factor rows over this kernel's grid sizes.
+        auto block_limit = [&](int t_r, const int4& ti, int u_r, const float4& ui) {
+            return block_limit_of(ct, w, simple, t_r, ti, u_r, ui);
+        };
+        // ---- by B* (lane = B* - 1): this kernel's grid sizes as places in the row's increasing order, and the
+        // row's minimum over them, the first place's.
         const bool g_dense = gm == g_ok;
+        const unsigned all_places = 0x10000u - (0x10000u >> x.n_g);
         if (lane == 0) w.iparmin[0] = __int_as_float(0x7fc00000);  // B* = 0: no valid configuration
         if (lane < kMaxB) {
             if (g_dense) {
                 w.iparmin[lane + 1] = ct.iparmin[lane];
             } else {
-                // the kernel's nG grid sizes only (a warp-uniform trip count)
-                const float* row = ct.ipar[lane];
-                float mn = kInf;
-                for (int j = 0; j < nG; ++j) mn = fminf(mn, row[w.gpos[j]]);
-                w.iparmin[lane + 1] = mn;
+                // (a warp-uniform trip count)
+                unsigned pl = 0;
+                const unsigned long long of = ct.place[lane];
+                for (int j = 0; j < nG; ++j) pl |= 1u << ((unsigned)(of >> (4 * w.gpos[j])) & 15u);
+                w.places[lane + 1] = (unsigned short)pl;
+                w.iparmin[lane + 1] = ct.ipar[lane][ct.rperm[lane][31 - __clz(pl)]];
             }
         }
         __syncwarp();
@@ -385,47 +423,41 @@ __global__ void __maxnreg__(64)
         int tau_i = -1;
         float tau0 = kInf;   // bound from the pre-pass
 
-        // Merge: each candidate lane walks its triple's grid sizes in increasing
-        // cost (the order of X * ipar(B*, G) over G depends on B* only); the warp
-        // repeatedly takes the smallest head and inserts it while it beats the k-th
+        // A lane's walk over the grid sizes of its candidate triple in increasing cost (the order of
+        // X * ipar(B*, G) over G depends on B* only): the highest set bit of `places` is the next one. Points
+        // are numbered t rank << 9 | g position << 5 | (u, c) rank, which orders them as their canonical
+        // indices do. (Scanning the row for the kernel's grid sizes instead: 317,078 kernels of 128 points,
+        // k = 15, 1,267 us against 741.)
+        struct Head {
+            float c;
+            int i;
+        };
+        auto peek = [&](unsigned places, int B, float X, int base) -> Head {
+            const int Bv = max(B, 1) - 1;  // (lanes without a triple have no places, and B* = 0)
+            const int g = ct.rperm[Bv][(31 - __clz(places | 1u))];
+            return {places ? __fmul_rn(X, ct.ipar[Bv][g]) : kInf, places ? base | (g << 5) : 0x7fffffff};
+        };
+        auto drop = [&](unsigned places) { return places & ~(0x80000000u >> __clz(places | 1u)); };
+
+        // Merge: the warp repeatedly takes the smallest head and inserts it while it beats the k-th
         // entry. A lane's walk is in (cost, index) order unless two nearly equal
         // ipar values round to one cost, or X underflows; then (relaxed) equal
         // costs are walked on until a head costs more than the k-th entry.
-        auto merge = [&](bool any, int B, float X, int base) {
-            const bool relaxed = !ct.order_safe || __any_sync(kFull, any && !(X >= 0x1p-100f));
-            int r = 0;
-            float hc = kInf;
-            int hi = 0x7fffffff;
-            auto advance = [&]() {
-                hc = kInf;
-                hi = 0x7fffffff;
-                if (g_dense) {  // every axis grid size present: rank = position
-                    if (r < x.n_g) {
-                        const int g = ct.perm[B - 1][r++];
-                        hc = __fmul_rn(X, ct.ipar[B - 1][g]);
-                        hi = base + g * nUC;
-                    }
-                    return;
-                }
-                while (r < x.n_g) {
-                    const int g = ct.perm[B - 1][r++];
-                    if ((gm >> g) & 1u) {
-                        hc = __fmul_rn(X, ct.ipar[B - 1][g]);
-                        hi = base + __popc(gm & ((1u << g) - 1u)) * nUC;
-                        break;
-                    }
-                }
-            };
-            if (any) advance();
+        auto merge = [&](unsigned places, int B, float X, int base) {
+            const bool relaxed = !ct.order_safe || __any_sync(kFull, places != 0u && !(X >= 0x1p-100f));
+            Head h = peek(places, B, X, base);
             for (;;) {
-                const unsigned mc = __reduce_min_sync(kFull, __float_as_uint(hc));
+                const unsigned mc = __reduce_min_sync(kFull, __float_as_uint(h.c));
                 const float mcf = __uint_as_float(mc);
-                const unsigned mi = __reduce_min_sync(kFull, hc == mcf ? (unsigned)hi : 0xffffffffu);
+                const unsigned mi = __reduce_min_sync(kFull, h.c == mcf ? (unsigned)h.i : 0xffffffffu);
                 if (mc >= 0x7f800000u || mcf > tau0 || mcf > tau_c) break;
                 const bool enters = key_less(mcf, (int)mi, tau_c, tau_i);
                 if (!enters && !relaxed) break;
                 if (enters) warp_list_insert(lc, li, tau_c, tau_i, mcf, (int)mi, k, lane);
-                if (hc == mcf && hi == (int)mi) advance();
+                if (h.c == mcf && h.i == (int)mi) {
+                    places = drop(places);
+                    h = peek(places, B, X, base);
+                }
             }
         };
 
@@ -473,20 +505,32 @@ __global__ void __maxnreg__(64)
                     const int4 ti = w.tinfo[t_r];
                     const int wb = ti.x;
                     const float ln = __int_as_float(ti.y);
-                    const int gwr = block_limit(t_r, ti, u_r);
-                    const float cnm = w.cnm[u_r], cmv = w.cm[u_r];
+                    const float4 ui = w.uinfo[u_r];
+                    const int gwr = block_limit(t_r, ti, u_r, ui);
+                    const float cnm = ui.x, cmv = ui.y;
                     float key[NC];
                     float pm = kInf;
+                    // branch-free: a triple without a valid configuration (B* = 0) reads
+                    // hide[0] and iparmin[0] = NaN, so it is keyed NaN (never a
+                    // candidate, not counted in the bound); W* = B* W_B <= W_mp <= kMaxW
+                    // for a valid triple. X is finite (counts <= 2^40). Two carveouts at a
+                    // time with packed FP32 operations, each rounded as the scalar ones.
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        // branch-free: a triple without a valid configuration (B* = 0) reads
-                        // hide[0] and iparmin[0] = NaN, so it is keyed NaN (never a
-                        // candidate, not counted in the bound); W* = B* W_B <= W_mp <= kMaxW
-                        // for a valid triple. X is finite (counts <= 2^40).
-                        const int B = min(gwr, gs[c]);
+                    for (int c = 0; c + 1 < NC; c += 2) {
+                        const int B0 = min(gwr, gs[c]), B1 = min(gwr, gs[c + 1]);
+                        const float2 X = mul2(fma2(make_float2(cmv, cmv), make_float2(ct.hide[B0 * wb], ct.hide[B1 * wb]),
+                                                   make_float2(cnm, cnm)),
+                                              make_float2(ln, ln));
+                        const float2 kk = mul2(X, make_float2(w.iparmin[B0], w.iparmin[B1]));
+                        key[c] = kk.x;
+                        key[c + 1] = kk.y;
+                        pm = fminf(pm, fminf(kk.x, kk.y));
+                    }
+                    if constexpr (NC & 1) {
+                        const int B = min(gwr, gs[NC - 1]);
                         const float X = __fmul_rn(__fmaf_rn(cmv, ct.hide[B * wb], cnm), ln);
-                        key[c] = __fmul_rn(X, w.iparmin[B]);
-                        pm = fminf(pm, key[c]);
+                        key[NC - 1] = __fmul_rn(X, w.iparmin[B]);
+                        pm = fminf(pm, key[NC - 1]);
                     }
                     int mult = 0;
 #pragma unroll
@@ -516,16 +560,15 @@ __global__ void __maxnreg__(64)
                 default: pairs(IntC<4>{}); break;
             }
             __syncwarp();
-            // entries in increasing order until they count k triples (at most 64 rounds; a
+            // entries in increasing order, equal ones at once, until they count k triples (a
             // finite entry counts at least one triple; +inf: fewer than k valid triples)
             for (int need = k;;) {
                 const unsigned mb = __reduce_min_sync(kFull, __float_as_uint(m0));
                 tau0 = __uint_as_float(mb);
                 if (mb >= 0x7f800000u) break;
-                const int src = __ffs(__ballot_sync(kFull, __float_as_uint(m0) == mb)) - 1;
-                need -= __shfl_sync(kFull, c0, src);
+                const bool me = __float_as_uint(m0) == mb;  // the lanes whose smallest is taken
+                need -= __reduce_add_sync(kFull, me ? c0 : 0);
                 if (need <= 0) break;
-                const bool me = lane == src;  // the lane whose smallest was taken
                 m0 = me ? m1 : m0;
                 c0 = me ? c1 : c0;
                 m1 = me ? kInf : m1;
@@ -544,12 +587,17 @@ __global__ void __maxnreg__(64)
                 const unsigned m = (kv.x <= tau0 ? 1u : 0u) | (kv.y <= tau0 ? 2u : 0u) |
                                    (kv.z <= tau0 ? 4u : 0u) | (kv.w <= tau0 ? 8u : 0u);
                 if (__ballot_sync(kFull, m != 0u) == 0u) continue;
+                // in triple order: those of the lanes before, then this lane's
+                int at = n_cand;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const unsigned bj = __ballot_sync(kFull, (m >> j) & 1u);
-                    if ((m >> j) & 1u) w.key[n_cand + __popc(bj & below)] = __int_as_float(t0 + j);
+                    at += __popc(bj & below);
                     n_cand += __popc(bj);
                 }
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if ((m >> j) & 1u) w.key[at++] = __int_as_float(t0 + j);
             }
             __syncwarp();
 
@@ -561,6 +609,7 @@ __global__ void __maxnreg__(64)
             for (int c0 = 0; c0 < n_cand; c0 += 32) {
                 const bool has = c0 + lane < n_cand;
                 int B = 0, base = 0;
+                unsigned places = 0;
                 float X = 0.0f;
                 if (has) {
                     const int tri = __float_as_int(w.key[c0 + lane]);
@@ -569,105 +618,63 @@ __global__ void __maxnreg__(64)
                     const int u_r = small_div(uc_r, rcp_c);
                     const int c = uc_r - u_r * nC;
                     const int4 ti = w.tinfo[t_r];
-                    B = min(block_limit(t_r, ti, u_r), w.gs[c]);
-                    X = __fmul_rn(__fmaf_rn(w.cm[u_r], ct.hide[B * ti.x], w.cnm[u_r]), __int_as_float(ti.y));
-                    base = t_r * g_stride + uc_r;
+                    const float4 ui = w.uinfo[u_r];
+                    B = min(block_limit(t_r, ti, u_r, ui), w.gs[c]);
+                    X = __fmul_rn(__fmaf_rn(ui.y, ct.hide[B * ti.x], ui.x), __int_as_float(ti.y));
+                    base = t_r << 9 | uc_r;
+                    places = g_dense ? all_places : w.places[B];
                 }
                 if (c0 > 0) {
-                    merge(has, B, X, base);
+                    merge(places, B, X, base);
                     continue;
                 }
-                int rg = 0;
-                float hc = kInf;
-                int hi = 0x7fffffff;
-                auto advance = [&]() {
-                    if (g_dense) {  // every axis grid size present: rank = position
-                        if (rg < x.n_g) {
-                            const int g = ct.perm[B - 1][rg++];
-                            hc = __fmul_rn(X, ct.ipar[B - 1][g]);
-                            hi = base + g * nUC;
-                        } else {
-                            hc = kInf;
-                            hi = 0x7fffffff;
-                        }
-                        return;
-                    }
-                    hc = kInf;
-                    hi = 0x7fffffff;
-                    while (rg < x.n_g) {
-                        const int g = ct.perm[B - 1][rg++];
-                        if ((gm >> g) & 1u) {
-                            hc = __fmul_rn(X, ct.ipar[B - 1][g]);
-                            hi = base + __popc(gm & ((1u << g) - 1u)) * nUC;
-                            break;
-                        }
-                    }
-                };
-                if (has) advance();
+                Head h = peek(places, B, X, base);
                 const bool relaxed = !ct.order_safe || __any_sync(kFull, has && !(X >= 0x1p-100f));
                 if (!relaxed) {
                     // every lane's walk is in (cost, index) order: the r-th extraction is the
                     // r-th best of the batch (points above tau0 cannot be among the top k)
-                    for (int r = 0; r < k;) {
-                        const unsigned mc = __reduce_min_sync(kFull, __float_as_uint(hc));
+                    // (w.iparmin is free after the scan: list position r, then read by lane r)
+                    float2* const list = reinterpret_cast<float2*>(w.iparmin);
+                    int r = 0;
+                    while (r < k) {
+                        const unsigned mc = __reduce_min_sync(kFull, __float_as_uint(h.c));
                         const float mcf = __uint_as_float(mc);
                         if (mc >= 0x7f800000u || mcf > tau0) break;
-                        const bool tie = hc == mcf;
-                        if (g_dense) {
-                            // every lane's next head, straight-line (B and the position are
-                            // clamped into range for lanes without one)
-                            const int Bv = max(B, 1) - 1;
-                            const int g = ct.perm[Bv][min(rg, x.n_g - 1)];
-                            const bool more = rg < x.n_g;
-                            const float nc = more ? __fmul_rn(X, ct.ipar[Bv][g]) : kInf;
-                            const int ni = more ? base + g * nUC : 0x7fffffff;
-                            // Heads of the smallest cost whose index is below every equal-cost
-                            // next head are the next points in (cost, index) order, all of them
-                            // (each walk is in that order). Where their indices rise with the
-                            // lane, as they mostly do (candidates are in triple order), the
-                            // first m go to list positions r.. at once through shared memory.
-                            const unsigned bound =
-                                __reduce_min_sync(kFull, tie && nc == mcf ? (unsigned)ni : 0xffffffffu);
-                            const bool elig = tie && (unsigned)hi < bound;
-                            const unsigned before = __ballot_sync(kFull, elig) & below;
-                            const int hprev = __shfl_sync(kFull, hi, before ? 31 - __clz(before) : lane);
-                            if (__all_sync(kFull, !elig || !before || hprev < hi)) {
-                                const int m = min(__popc(__ballot_sync(kFull, elig)), k - r);
-                                const int rank = __popc(before);
-                                const bool take = elig && rank < m;
-                                // w.iparmin is free during the selection: [j] cost, [16 + j] index
-                                if (take) {
-                                    w.iparmin[rank] = hc;
-                                    w.iparmin[16 + rank] = __int_as_float(hi);
-                                }
-                                __syncwarp();
-                                if (lane >= r && lane < r + m) {
-                                    lc = w.iparmin[lane - r];
-                                    li = __float_as_int(w.iparmin[16 + lane - r]);
-                                }
-                                __syncwarp();
-                                hc = take ? nc : hc;
-                                hi = take ? ni : hi;
-                                rg += take ? 1 : 0;
-                                r += m;
-                                continue;
-                            }
+                        const bool tie = h.c == mcf;
+                        // every lane's next head, straight-line
+                        const unsigned rest = drop(places);
+                        const Head nx = peek(rest, B, X, base);
+                        // Heads of the smallest cost whose index is below every equal-cost
+                        // next head are the next points in (cost, index) order, all of them
+                        // (each walk is in that order). Where their indices rise with the
+                        // lane, as they mostly do (candidates are in triple order), the
+                        // first ones go to list positions r.. at once.
+                        const unsigned bound =
+                            __reduce_min_sync(kFull, tie && nx.c == mcf ? (unsigned)nx.i : 0xffffffffu);
+                        const bool elig = tie && (unsigned)h.i < bound;
+                        const unsigned eb = __ballot_sync(kFull, elig), before = eb & below;
+                        const int hprev = __shfl_sync(kFull, h.i, before ? 31 - __clz(before) : lane);
+                        bool take;
+                        if (__all_sync(kFull, !elig || !before || hprev < h.i)) {
+                            const int to = r + __popc(before);
+                            take = elig && to < k;
+                            if (take) list[to] = make_float2(h.c, __int_as_float(h.i));
+                            r += __popc(eb);
+                        } else {
                             // indices out of lane order: one point, the lowest index
-                            const unsigned mi = __reduce_min_sync(kFull, tie ? (unsigned)hi : 0xffffffffu);
-                            lc = lane == r ? mcf : lc;
-                            li = lane == r ? (int)mi : li;
-                            const bool win = tie && hi == (int)mi;
-                            hc = win ? nc : hc;
-                            hi = win ? ni : hi;
-                            rg += win ? 1 : 0;
+                            const unsigned mi = __reduce_min_sync(kFull, tie ? (unsigned)h.i : 0xffffffffu);
+                            take = tie && h.i == (int)mi;
+                            if (take) list[r] = make_float2(h.c, __int_as_float(h.i));
                             ++r;
-                            continue;
                         }
-                        const unsigned mi = __reduce_min_sync(kFull, tie ? (unsigned)hi : 0xffffffffu);
-                        lc = lane == r ? mcf : lc;
-                        li = lane == r ? (int)mi : li;
-                        if (tie && hi == (int)mi) advance();
-                        ++r;
+                        if (take) h = nx;
+                        places = take ? rest : places;
+                    }
+                    __syncwarp();
+                    if (lane < min(r, k)) {
+                        const float2 e = list[lane];
+                        lc = e.x;
+                        li = __float_as_int(e.y);
                     }
                     tau_c = __shfl_sync(kFull, lc, k - 1);
                     tau_i = __shfl_sync(kFull, li, k - 1);
@@ -677,10 +684,10 @@ __global__ void __maxnreg__(64)
                 float prev_c = 0.0f;
                 int prev_i = -1;
                 for (;;) {
-                    const unsigned mc = __reduce_min_sync(kFull, __float_as_uint(hc));
+                    const unsigned mc = __reduce_min_sync(kFull, __float_as_uint(h.c));
                     const float mcf = __uint_as_float(mc);
                     if (mc >= 0x7f800000u || mcf > tau0 || mcf > tau_c) break;
-                    const unsigned mi = __reduce_min_sync(kFull, hc == mcf ? (unsigned)hi : 0xffffffffu);
+                    const unsigned mi = __reduce_min_sync(kFull, h.c == mcf ? (unsigned)h.i : 0xffffffffu);
                     if (cnt == k && !relaxed && !key_less(mcf, (int)mi, tau_c, tau_i)) break;
                     if (cnt < k && (cnt == 0 || key_less(prev_c, prev_i, mcf, (int)mi))) {
                         if (lane == cnt) {  // in order: append
@@ -701,12 +708,17 @@ __global__ void __maxnreg__(64)
                             tau_i = __shfl_sync(kFull, li, k - 1);
                         }
                     }
-                    if (hc == mcf && hi == (int)mi) advance();
+                    if (h.c == mcf && h.i == (int)mi) {
+                        places = drop(places);
+                        h = peek(places, B, X, base);
+                    }
                 }
             }
         }
         if (lane < k) {
-            topk_idx[kid * k + lane] = li;
+            const int g = (li >> 5) & 15;  // the canonical index of the numbered point
+            const int at = (li >> 9) * g_stride + __popc(gm & ((1u << g) - 1u)) * nUC + (li & 31);
+            topk_idx[kid * k + lane] = li < 0 ? -1 : at;
             topk_cost[kid * k + lane] = lc;
         }
         __syncwarp();  // the warp's tables are rewritten for the next descriptor
@@ -965,7 +977,7 @@ __global__ void __maxnreg__(KMAX > 8 ? 128 : 96)
                     // grid sizes in increasing cost: the order of ipar(B*, G) over G
 #pragma unroll 1
                     for (int r = 0; r < x.n_g; ++r) {
-                        const int g = ct.perm[B - 1][r];
+                        const int g = ct.rperm[B - 1][15 - r];
                         const float cg = __fmul_rn(X, ct.ipar[B - 1][g]);
                         if (cg > fminf(thr_c, tau0)) break;
                         const int idx = base + g * nUC;
@@ -1022,11 +1034,11 @@ int launch_thread(const EvalParams& p, const tune_kernel_desc* descs, int32_t* t
     return TUNE_OK;
 }
 
-// One row's launch; `dependent`: it may start while the launch before it, another row's, still runs.
+// One row's launch of `rows`; `dependent`: it may start while the launch before it, another row's, still runs.
 template <bool EMIT>
 int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, float* tc, int32_t* pb, int32_t* pw,
            float* pc, const int64_t* po, int* status, cudaStream_t s, int ctas_per_sm = 0,
-           unsigned long long* queue = nullptr, bool dependent = false)
+           unsigned long long* queue = nullptr, bool dependent = false, int rows = 1)
 {
     auto kern = tune_eval_kernel<EMIT>;
     static std::atomic<int> per_sm_cache[tune::kMaxDevices];
@@ -1036,7 +1048,11 @@ int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, floa
     const int sms = tune::device_sm_count();
     if (sms <= 0) return tune::fail(TUNE_ECUDA, "tune_eval: cannot query the SM count");
     const int64_t need = (p.n_kernels + kWarps - 1) / kWarps;
-    const int64_t cap = (int64_t)sms * (ctas_per_sm > 0 ? min(ctas_per_sm, per_sm) : per_sm);
+    int64_t cap = (int64_t)sms * (ctas_per_sm > 0 ? min(ctas_per_sm, per_sm) : per_sm);
+    // Where a row has fewer than two descriptors per warp of a full grid, the rows share the chip side by side
+    // instead (4,574 dense kernels against six rows: 94 -> 85 us; 18,548 against five, 3.8 per warp: 199 us row
+    // by row, 255 side by side).
+    if (rows > 1 && need < 2 * cap) cap = (cap + rows - 1) / rows;
     const int grid = (int)std::min(EMIT ? p.n_kernels : need, cap);
     // By default the queue counter follows the status word in the zeroed workspace header.
     if (!queue) queue = reinterpret_cast<unsigned long long*>(status) + 1;
@@ -1289,7 +1305,7 @@ extern "C" int tune_eval_archs(const tune_arch* archs, int32_t n_arch, const tun
     if (n_kernels == 0) return TUNE_OK;
     // A launch per row, with the row's tables from the host, each starting in the places that the one before it
     // leaves. (One launch for all rows, whose CTAs built their row's tables and read its fields by a row
-    // index: 519 us for 50,000 uneven kernels against six rows; now 493.)
+    // index: 519 us for 50,000 uneven kernels against six rows; now 430.)
     EvalParams p;
     p.x = *axes;
     p.n_kernels = n_kernels;
@@ -1299,7 +1315,7 @@ extern "C" int tune_eval_archs(const tune_arch* archs, int32_t n_arch, const tun
         p.a = archs[i];
         const int64_t at = (int64_t)i * n_kernels * k;
         const int rc = launch<false>(p, descs, topk_idx + at, topk_cost + at, nullptr, nullptr, nullptr, nullptr, status, s,
-                                     (int)((flags >> 12) & 0xfu), reinterpret_cast<unsigned long long*>(status) + 1 + i, i > 0);
+                                     (int)((flags >> 12) & 0xfu), reinterpret_cast<unsigned long long*>(status) + 1 + i, i > 0, n_arch);
         if (rc) return rc;
     }
     return TUNE_OK;
