@@ -746,23 +746,36 @@ __global__ void __maxnreg__(64)
         // warps write each one's points, an eighth of the thread counts each: the spaces' sizes differ, and a warp
         // by itself needs 25 us for the points of a full one. (20,000 uneven kernels, 114 M points: 534 us with a
         // warp per descriptor, lanes on triples and each lane writing its grid sizes nUC points apart; 316 with
-        // the points written in order; 281 shared by the CTA, the HBM floor being 201; 6,000 dense ones: 226 -> 181,
+        // the points written in order; 281 shared by the CTA, the HBM floor being 201 (253 now, see below); 6,000 dense ones: 226 -> 181,
         // 0.96 of the HBM rate.)
+        // Towards the end of the descriptors the groups shrink, to as few as have about 16,384 points (by the mean
+        // of the offsets), so that no CTA is left with eight large spaces: 280 -> 253 us.
         __shared__ long long next;
+        __shared__ int next_size;
         const int warp = threadIdx.x >> 5;
-        const int64_t groups = (n_k + p.group - 1) / p.group;
-        for (int64_t g = blockIdx.x; g < groups;) {
-            if (threadIdx.x == 0) next = (long long)gridDim.x + (long long)atomicAdd(queue, 1ull);
-            const int64_t kid = g * p.group + warp;
+        int least = 1;
+        if (threadIdx.x == 0) {
+            const int64_t mean = n_k > 1 ? max((int64_t)1, (pt_off[n_k - 1] - pt_off[0]) / (n_k - 1)) : 1;
+            least = (int)max((int64_t)1, min((int64_t)kWarps, 16384 / mean));
+        }
+        int size = p.group;
+        for (int64_t g = (int64_t)blockIdx.x * size; g < n_k;) {
+            if (threadIdx.x == 0) {
+                const int64_t even = (n_k - g) / (4 * (int64_t)gridDim.x);
+                next_size = min(p.group, (int)max((int64_t)least, min((int64_t)kWarps, even)));
+                next = (long long)gridDim.x * p.group + (long long)atomicAdd(queue, (unsigned long long)next_size);
+            }
+            const int64_t kid = g + warp;
             if (lane == 0) w.nT = 0;
             __syncwarp();
-            if (warp < p.group && kid < n_k) rank(kid, __ldg(descs + kid * 4 + (lane & 3)));
+            if (warp < size && kid < n_k) rank(kid, __ldg(descs + kid * 4 + (lane & 3)));
             __syncthreads();
-            for (int i = 0; i < p.group; ++i) {
+            for (int i = 0; i < size; ++i) {
                 const WarpTables& t = wts[i];
                 emit_points(ct, t, w.tri, warp * t.nT / kWarps, (warp + 1) * t.nT / kWarps, lane, pt_b, pt_w, pt_c);
             }
             g = next;
+            size = next_size;
             __syncthreads();  // the tables and `next` are rewritten
         }
         return;
