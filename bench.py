@@ -84,9 +84,9 @@ def triple_instructions(descs):
 
 
 def kernel_source_hash():
-    """Hash of the evaluation kernel's sources (tune_eval.cu and the arithmetic it includes)."""
+    """Hash of the evaluation kernel's sources (tune_eval.cu, the arithmetic and tables it includes)."""
     h = hashlib.sha256()
-    for name in ("tune_eval.cu", "eval_common.cuh"):
+    for name in ("tune_eval.cu", "eval_common.cuh", "eval_tables.cuh", "eval_tables.cu"):
         with open(os.path.join(ROOT, "paper_1701_08547_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -722,9 +722,9 @@ def train_section(args, dev, data, members, peaks, stream):
                     "call": "features, labels and epoch orders copied from pinned host memory, surrogate_train, "
                             "loss trace copied back, all inside the timed region"},
             "final_mse": float(trace[-1].mean()),
-            # per step: batch gather, fused forward, loss (2), head backward (2), weight transpose and
-            # fused input-gradient chain (2), four weight-gradient passes with their reductions (8), Adam
-            "gpu_launches": 17 * epochs * steps}
+            # per step: fused forward, head backward, fused input-gradient chain, weight gradients, Adam (with
+            # the next batch's gather); the first batch's gather
+            "gpu_launches": 1 + 5 * epochs * steps}
     if not args.no_cpu_baseline:
         line["cpu_baseline"] = train_cpu_baseline(members)
     return line, sur
