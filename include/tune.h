@@ -185,8 +185,9 @@ int tune_eval(const tune_arch* arch, const tune_axes* axes, const tune_kernel_de
  *    device's primary context: after cudaDeviceReset (or anything else that
  *    destroys and recreates that context) it is stale, so do not use this
  *    entry point across a device reset.
- *  - Every call shares the array and clears the part it uses at the start;
- *    calls that overlap on the GPU (for example on two streams) race on it.
+ *  - A call has a 256-byte header of the array to itself until it returns, so
+ *    calls on several streams and host threads do not disturb each other; at
+ *    most 16 are under way on a device, a further one waits for one of them.
  *  - The call waits for `stream` before returning, so that it can return
  *    TUNE_EINVAL for malformed descriptors found by the kernel.
  */

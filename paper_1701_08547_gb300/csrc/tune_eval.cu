@@ -37,6 +37,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <condition_variable>
 #include <limits>
 #include <mutex>
 
@@ -1205,28 +1206,78 @@ namespace {
 
 constexpr size_t kNoallocScratchBytes = 4096;  // stated maximum scratch for one call
 
-// Scratch of tune_eval_noalloc (status word and counters). Shared by every
-// call on a device: calls that overlap on the GPU race on it.
+// Scratch of tune_eval_noalloc: a header (status word and the emitting pass's queue) per call under way. Calls
+// that shared one would take descriptor groups from each other's queue and leave points unwritten.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+constexpr int kNoallocHeaders = (int)(kNoallocScratchBytes / tune::kWorkspaceHeader);
+static_assert(kNoallocHeaders <= 32, "a bit per header");
 
-std::mutex g_noalloc_mu;
-void* g_noalloc_ptr[tune::kMaxDevices] = {nullptr};
+struct NoallocDevice {
+    std::mutex mu;
+    std::condition_variable freed;
+    char* base = nullptr;  // device address of the array, looked up once
+    uint32_t busy = 0;     // headers in use
+};
+NoallocDevice g_noalloc[tune::kMaxDevices];
 
-// Device address of the scratch array for the current device, looked up once
-// per device (host code must not use the symbol itself: on the host it names a
-// stand-in object, not device memory).
-int noalloc_scratch(void** out)
-{
-    int dev = 0;
-    TUNE_CUDA_TRY(cudaGetDevice(&dev), "tune_eval_noalloc: cudaGetDevice");
-    if (dev < 0 || dev >= tune::kMaxDevices) return tune::fail(TUNE_EUNSUPPORTED, "device ordinal %d too large", dev);
-    std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    if (!g_noalloc_ptr[dev]) {
-        void* p = nullptr;
-        TUNE_CUDA_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch), "tune_eval_noalloc: cudaGetSymbolAddress");
-        g_noalloc_ptr[dev] = p;
+// One of the current device's headers, the caller's until the object goes (waits while all are taken).
+class NoallocHeader {
+public:
+    ~NoallocHeader()
+    {
+        if (!ptr_) return;
+        std::lock_guard<std::mutex> lock(dev_->mu);
+        dev_->busy &= ~(1u << slot_);
+        dev_->freed.notify_one();
     }
-    *out = g_noalloc_ptr[dev];
+    // (Host code must not use the array's symbol itself: on the host it names a stand-in object, not device memory.)
+    int take(void** out)
+    {
+        int dev = 0;
+        TUNE_CUDA_TRY(cudaGetDevice(&dev), "tune_eval_noalloc: cudaGetDevice");
+        if (dev < 0 || dev >= tune::kMaxDevices) return tune::fail(TUNE_EUNSUPPORTED, "device ordinal %d too large", dev);
+        dev_ = &g_noalloc[dev];
+        std::unique_lock<std::mutex> lock(dev_->mu);
+        if (!dev_->base) {
+            void* p = nullptr;
+            TUNE_CUDA_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch), "tune_eval_noalloc: cudaGetSymbolAddress");
+            dev_->base = static_cast<char*>(p);
+        }
+        constexpr uint32_t all = (uint32_t)((1ull << kNoallocHeaders) - 1);
+        dev_->freed.wait(lock, [&] { return dev_->busy != all; });
+        slot_ = __builtin_ctz(~dev_->busy);
+        dev_->busy |= 1u << slot_;
+        ptr_ = *out = dev_->base + slot_ * tune::kWorkspaceHeader;
+        return TUNE_OK;
+    }
+
+private:
+    NoallocDevice* dev_ = nullptr;
+    void* ptr_ = nullptr;
+    int slot_ = 0;
+};
+
+// The call on its header: everything that uses it is complete when this returns TUNE_OK.
+int noalloc_call(void* scratch, EvalParams& p, const tune_kernel_desc* descs, bool emit, int32_t* topk_idx, float* topk_cost,
+                 int32_t* pt_blocks, int32_t* pt_warps, float* pt_cost, const int64_t* pt_offsets, cudaStream_t s)
+{
+    // The array keeps earlier calls' contents: clear the status word and counters.
+    TUNE_CUDA_TRY(cudaMemsetAsync(scratch, 0, tune::kWorkspaceHeader, s), "tune_eval_noalloc: scratch reset");
+    if (p.n_kernels > 0) {
+        int* status = static_cast<int*>(scratch);
+        const int rc = emit ? launch<true>(p, descs, topk_idx, topk_cost, pt_blocks, pt_warps, pt_cost, pt_offsets, status, s)
+                            : launch<false>(p, descs, topk_idx, topk_cost, nullptr, nullptr, nullptr, nullptr, status, s);
+        if (rc) return rc;
+    }
+    // Report what the kernel found: wait for the stream and read the status word.
+    int st = 0;
+    TUNE_CUDA_TRY(cudaMemcpyAsync(&st, scratch, sizeof(int), cudaMemcpyDeviceToHost, s),
+                  "tune_eval_noalloc: status read");
+    TUNE_CUDA_TRY(cudaStreamSynchronize(s), "tune_eval_noalloc: cudaStreamSynchronize");
+    if (st & tune::kStatusTimeout) return tune::fail(TUNE_ETIMEOUT, "a bounded device-side wait gave up");
+    if (st & tune::kStatusInvalid)
+        return tune::fail(TUNE_EINVAL, "a descriptor was malformed (mask outside the axes, negative "
+                                       "count, register or shared-memory field)");
     return TUNE_OK;
 }
 
@@ -1256,34 +1307,20 @@ extern "C" int tune_eval_noalloc(const tune_arch* arch, const tune_axes* axes,
     const bool emit = (flags & TUNE_EMIT_POINTS) != 0;
     if (emit && !pt_offsets) return tune::fail(TUNE_EINVAL, "TUNE_EMIT_POINTS needs pt_offsets");
 
+    NoallocHeader header;
     void* scratch = nullptr;
-    rc = noalloc_scratch(&scratch);
+    rc = header.take(&scratch);
     if (rc) return rc;
+    EvalParams p;
+    p.a = *arch;
+    p.x = *axes;
+    p.n_kernels = n_kernels;
+    p.k = k;
+    p.chunk = 0;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // The array keeps the previous call's contents: clear the status word and counters.
-    TUNE_CUDA_TRY(cudaMemsetAsync(scratch, 0, tune::kWorkspaceHeader, s), "tune_eval_noalloc: scratch reset");
-    if (n_kernels > 0) {
-        EvalParams p;
-        p.a = *arch;
-        p.x = *axes;
-        p.n_kernels = n_kernels;
-        p.k = k;
-        p.chunk = 0;
-        int* status = static_cast<int*>(scratch);
-        rc = emit ? launch<true>(p, descs, topk_idx, topk_cost, pt_blocks, pt_warps, pt_cost, pt_offsets, status, s)
-                  : launch<false>(p, descs, topk_idx, topk_cost, nullptr, nullptr, nullptr, nullptr, status, s);
-        if (rc) return rc;
-    }
-    // Report what the kernel found: wait for the stream and read the status word.
-    int st = 0;
-    TUNE_CUDA_TRY(cudaMemcpyAsync(&st, scratch, sizeof(int), cudaMemcpyDeviceToHost, s),
-                  "tune_eval_noalloc: status read");
-    TUNE_CUDA_TRY(cudaStreamSynchronize(s), "tune_eval_noalloc: cudaStreamSynchronize");
-    if (st & tune::kStatusTimeout) return tune::fail(TUNE_ETIMEOUT, "a bounded device-side wait gave up");
-    if (st & tune::kStatusInvalid)
-        return tune::fail(TUNE_EINVAL, "a descriptor was malformed (mask outside the axes, negative "
-                                       "count, register or shared-memory field)");
-    return TUNE_OK;
+    rc = noalloc_call(scratch, p, descs, emit, topk_idx, topk_cost, pt_blocks, pt_warps, pt_cost, pt_offsets, s);
+    if (rc) cudaStreamSynchronize(s);  // the header goes to the next call with nothing of this one under way
+    return rc;
 }
 
 // ---------------------------------------------------------------------------
