@@ -150,8 +150,8 @@ enum { TUNE_CALL_EVAL = 0, TUNE_CALL_TOPK = 1 };
  *   sizes. Invalid points get B* = W* = 0, cost = +inf. Any of the three may
  *   be NULL.
  * Arguments: arch, axes (host); descs (device, 16-byte aligned,
- * n_kernels records); 1 <= k <= 16; workspace (device) of at least
- * tune_workspace_bytes(TUNE_CALL_EVAL, n_kernels, k) bytes.
+ * n_kernels records); 1 <= k <= 16; workspace (device, 4-byte aligned) of at
+ * least tune_workspace_bytes(TUNE_CALL_EVAL, n_kernels, k) bytes.
  * n_kernels = 0 is valid and enqueues only the status reset.
  * A malformed descriptor (mask selecting values outside the axes, or a
  * field outside its range: a count above 2^40, negative or not a number,

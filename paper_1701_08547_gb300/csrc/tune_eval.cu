@@ -1048,6 +1048,13 @@ int launch_thread(const EvalParams& p, const tune_kernel_desc* descs, int32_t* t
     return TUNE_OK;
 }
 
+// Queue counter `i` of a workspace header: the 8-byte words after the status word, wherever in memory the caller's
+// workspace begins (the ranking by default needs the status word's alignment only, the emitting pass always a queue).
+unsigned long long* queue_word(int* status, int i)
+{
+    return reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(status + 1) + 7) & ~uintptr_t(7)) + i;
+}
+
 // One row's launch of `rows`; `dependent`: it may start while the launch before it, another row's, still runs.
 template <bool EMIT>
 int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, float* tc, int32_t* pb, int32_t* pw,
@@ -1068,8 +1075,8 @@ int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, floa
     // by row, 255 side by side).
     if (rows > 1 && need < 2 * cap) cap = (cap + rows - 1) / rows;
     const int grid = (int)std::min(EMIT ? p.n_kernels : need, cap);
-    // By default the queue counter follows the status word in the zeroed workspace header.
-    if (!queue) queue = reinterpret_cast<unsigned long long*>(status) + 1;
+    // By default the first queue counter of the zeroed workspace header.
+    if (!queue) queue = queue_word(status, 0);
     EvalParams q = p;
     // emitting: as many descriptors at a time, up to one per warp, as leave each CTA about three turns (the queue
     // evens out spaces of different sizes)
@@ -1365,7 +1372,7 @@ extern "C" int tune_eval_archs(const tune_arch* archs, int32_t n_arch, const tun
         p.a = archs[i];
         const int64_t at = (int64_t)i * n_kernels * k;
         const int rc = launch<false>(p, descs, topk_idx + at, topk_cost + at, nullptr, nullptr, nullptr, nullptr, status, s,
-                                     (int)((flags >> 12) & 0xfu), reinterpret_cast<unsigned long long*>(status) + 1 + i, i > 0, n_arch);
+                                     (int)((flags >> 12) & 0xfu), queue_word(status, i), i > 0, n_arch);
         if (rc) return rc;
     }
     return TUNE_OK;
