@@ -319,7 +319,8 @@ int tune_features(const tune_arch* arch, const tune_axes* axes, const tune_kerne
  * pt_offsets_host: host int64 [n_kernels + 1], exclusive scan of space sizes
  * (each space <= 2^20 points). Outputs (device): topk_idx, topk_score
  * [n_kernels, k], used_fallback uint8 [n_kernels]. workspace of at least
- * surrogate_infer_workspace_bytes(members, n_kernels, k). Synchronous.
+ * surrogate_infer_workspace_bytes(members, n_kernels, k), 8-byte aligned (16-byte for the
+ * tcgen05 forwards, whose feature rows lie in it). Synchronous.
  */
 int surrogate_infer(tune_surrogate* h, const tune_arch* arch, const tune_axes* axes,
                     const tune_kernel_desc* descs, int64_t n_kernels, const int64_t* pt_offsets_host,

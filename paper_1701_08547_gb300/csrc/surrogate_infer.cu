@@ -236,6 +236,8 @@ __global__ void __launch_bounds__(32 * kFeatWarps, 7)
     row[6 ^ sx] = zero;
     row[7 ^ sx] = zero;
 
+    // rows start at 16-byte boundaries unless the caller's workspace does not
+    const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
     int64_t cur = -1, cur_beg = 0, cur_end = 0;  // the kernel of the tables and its points
     bool cur_bad = false, staged = false;        // staged: every row's units 0, 1 are cur's
     int size = 0, nC = 1, nU = 1, nG = 1;
@@ -356,11 +358,17 @@ __global__ void __launch_bounds__(32 * kFeatWarps, 7)
         __syncwarp();
         if (on) score[base + lane] = valid ? 0.0f : __int_as_float(0x7f800000);
         const int rows = (int)(end - base < 32 ? end - base : 32);
-        uint4* dst = reinterpret_cast<uint4*>(out + base * IN);
+        if (aligned) {
+            uint4* dst = reinterpret_cast<uint4*>(out + base * IN);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = i * 4 + (lane >> 3), j = lane & 7;
-            if (r < rows) dst[i * 32 + lane] = s.stage[r * 8 + (j ^ (r & 7))];
+            for (int i = 0; i < 8; ++i) {
+                const int r = i * 4 + (lane >> 3), j = lane & 7;
+                if (r < rows) dst[i * 32 + lane] = s.stage[r * 8 + (j ^ (r & 7))];
+            }
+        } else {  // a word of a row per lane
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(s.stage);
+            uint32_t* dst = reinterpret_cast<uint32_t*>(out + base * IN);
+            for (int r = 0; r < rows; ++r) dst[r * 32 + lane] = src[(r * 8 + ((lane >> 2) ^ (r & 7))) * 4 + (lane & 3)];
         }
         __syncwarp();  // the staged rows have been read
     }
