@@ -28,10 +28,12 @@ def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
     torch = _torch()
-    if not torch.cuda.is_initialized():
+    # (the handle without a Stream object around it, where this PyTorch gives it: 0.2 us instead of 3 per call)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    # (the handle without a Stream object around it: 0.2 us instead of 3 per call)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return raw(device())
 
 
 def _ptr(t):
