@@ -1,20 +1,25 @@
-// Programmatic dependent launch for the surrogate's training step.
+// Programmatic dependent launch.
 //
-// A training step is a chain of launches on one stream, each consuming the one
-// before it. Launched with the programmatic-serialization attribute, a kernel
-// may be scheduled while its predecessor is still running; its CTAs then park
-// in grid_dep_wait() until the predecessor has completed and its memory
-// operations are visible, so the launch latency between the two is hidden.
+// Launched with the programmatic-serialization attribute, a kernel may be scheduled while its predecessor on the
+// stream is still running: once every CTA of the predecessor has called grid_dep_launch() or left. grid_dep_wait()
+// returns when the predecessor has completed and its memory operations are visible. In a kernel launched without the
+// attribute both calls return at once. Two patterns are used:
 //
-// Rules that keep this correct and free of deadlock:
-//  * every kernel launched by launch_dep() calls grid_dep_wait() before any
-//    global-memory access (read or write) and before allocating tensor memory,
-//    except reads of data that no launch from its predecessor's predecessor on
-//    writes (that one is complete when the predecessor's CTAs start their
-//    successor);
-//  * a kernel calls grid_dep_launch() only after its own grid_dep_wait(), so at
-//    most one kernel waits ahead of the running one;
-//  * in a kernel launched without the attribute both calls return at once.
+// Chains (a training step of the surrogate): each kernel consumes what the one before it wrote. Its CTAs park in
+// grid_dep_wait(), which hides the launch latency.
+//  * every kernel of a chain calls grid_dep_wait() before any global-memory access (read or write) and before
+//    allocating tensor memory, except reads of data that no launch from its predecessor's predecessor on writes;
+//    that one is complete when the predecessor's CTAs start their successor, because
+//  * a kernel of a chain calls grid_dep_launch() only after its own grid_dep_wait(); so at most one kernel waits ahead
+//    of the running one, too.
+//
+// Independent launches (the rows of tune_eval_archs): kernels that read only what was written before the first of them
+// and whose outputs, counters included, are disjoint. The first is launched without the attribute. Each but the last
+// calls grid_dep_launch() at its start, so that the next one's CTAs take the places that its own leave, and every
+// thread of each calls grid_dep_wait() before it ends, so that a launch is complete only after all before it.
+//  * the last one does not call grid_dep_launch(): what follows it on the stream, a chain whose kernels read early
+//    among it, starts when all of them are complete.
+//  * a launch's CTAs start after all CTAs of the one before it have, so that waiting CTAs keep no place from them.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -64,6 +64,7 @@ struct EvalParams {
     int k;
     int chunk;        // dynamic work queue: kernels per grab (0 = each CTA its own descriptors)
     int group;        // emitting: descriptors a CTA takes at a time (1..8)
+    int next_row;     // another row of the same sweep is launched next
     CtaTables tab;
 };
 
@@ -303,7 +304,9 @@ __global__ void __maxnreg__(64)
     __shared__ WarpTables wts[kWarps];
     __shared__ int taken;
     const tune_arch& a = p.a;
-    pdl::grid_dep_launch();  // a row of tune_eval_archs: the next row's CTAs may take the places this one's leave
+    // a row of tune_eval_archs before the last: the next row's CTAs may take the places that this one's leave
+    // (independent launches, pdl.cuh)
+    if (p.next_row) pdl::grid_dep_launch();
     copy_cta_tables(p.tab, ct);
     if (threadIdx.x == 0) taken = kWarps;
     __syncthreads();
@@ -807,7 +810,7 @@ __global__ void __maxnreg__(64)
         kid = nk;
         v = v_next;
     }
-    pdl::grid_dep_wait();  // the launch is complete only after the row's before it
+    pdl::grid_dep_wait();  // a row is complete only after the row before it
 }
 
 // ---- thread-per-kernel schedule ---------------------------------------------
@@ -1055,11 +1058,11 @@ unsigned long long* queue_word(int* status, int i)
     return reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(status + 1) + 7) & ~uintptr_t(7)) + i;
 }
 
-// One row's launch of `rows`; `dependent`: it may start while the launch before it, another row's, still runs.
+// Row `row` of the `rows` of a sweep. Rows after the first may start while the one before them still runs.
 template <bool EMIT>
 int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, float* tc, int32_t* pb, int32_t* pw,
            float* pc, const int64_t* po, int* status, cudaStream_t s, int ctas_per_sm = 0,
-           unsigned long long* queue = nullptr, bool dependent = false, int rows = 1)
+           unsigned long long* queue = nullptr, int row = 0, int rows = 1)
 {
     auto kern = tune_eval_kernel<EMIT>;
     static std::atomic<int> per_sm_cache[tune::kMaxDevices];
@@ -1078,12 +1081,13 @@ int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, floa
     // By default the first queue counter of the zeroed workspace header.
     if (!queue) queue = queue_word(status, 0);
     EvalParams q = p;
+    q.next_row = row + 1 < rows;
     // emitting: as many descriptors at a time, up to one per warp, as leave each CTA about three turns (the queue
     // evens out spaces of different sizes)
     q.group = (int)std::max<int64_t>(1, std::min<int64_t>(kWarps, p.n_kernels / (3 * cap)));
     tune::eval_tables(q.a, q.x, q.tab);
     const int4* d = reinterpret_cast<const int4*>(descs);
-    if (dependent)
+    if (row > 0)
         TUNE_CUDA_TRY(pdl::launch_dep(kern, dim3(grid), dim3(kThreads), 0, s, q, d, ti, tc, pb, pw, pc, po, status, queue),
                       "tune_eval: kernel launch");
     else
@@ -1372,7 +1376,7 @@ extern "C" int tune_eval_archs(const tune_arch* archs, int32_t n_arch, const tun
         p.a = archs[i];
         const int64_t at = (int64_t)i * n_kernels * k;
         const int rc = launch<false>(p, descs, topk_idx + at, topk_cost + at, nullptr, nullptr, nullptr, nullptr, status, s,
-                                     (int)((flags >> 12) & 0xfu), queue_word(status, i), i > 0, n_arch);
+                                     (int)((flags >> 12) & 0xfu), queue_word(status, i), i, n_arch);
         if (rc) return rc;
     }
     return TUNE_OK;
