@@ -15,8 +15,8 @@
 //
 // Independent launches (the rows of tune_eval_archs): kernels that read only what was written before the first of them
 // and whose outputs, counters included, are disjoint. The first is launched without the attribute. Each but the last
-// calls grid_dep_launch() at its start, so that the next one's CTAs take the places that its own leave, and every
-// thread of each calls grid_dep_wait() before it ends, so that a launch is complete only after all before it.
+// calls grid_dep_launch() at its start, so that the next one's CTAs take the places that its own leave, and one CTA
+// of each calls grid_dep_wait() before it ends, so that a launch is complete only after all before it.
 //  * the last one does not call grid_dep_launch(): what follows it on the stream, a chain whose kernels read early
 //    among it, starts when all of them are complete.
 //  * a launch's CTAs start after all CTAs of the one before it have, so that waiting CTAs keep no place from them.

@@ -810,7 +810,9 @@ __global__ void __maxnreg__(64)
         kid = nk;
         v = v_next;
     }
-    pdl::grid_dep_wait();  // a row is complete only after the row before it
+    // A row is complete only after the row before it. One CTA waits: if all did, those that find the queue empty would
+    // keep their places from the rows after (9,800 dense kernels against six rows, 16 per grab: 658 us, now 288).
+    if (blockIdx.x == 0) pdl::grid_dep_wait();
 }
 
 // ---- thread-per-kernel schedule ---------------------------------------------
