@@ -1075,15 +1075,20 @@ int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, floa
     if (sms <= 0) return tune::fail(TUNE_ECUDA, "tune_eval: cannot query the SM count");
     const int64_t need = (p.n_kernels + kWarps - 1) / kWarps;
     int64_t cap = (int64_t)sms * (ctas_per_sm > 0 ? min(ctas_per_sm, per_sm) : per_sm);
-    // Where a row has fewer than two descriptors per warp of a full grid, the rows share the chip side by side
-    // instead (4,574 dense kernels against six rows: 94 -> 85 us; 18,548 against five, 3.8 per warp: 199 us row
-    // by row, 255 side by side).
-    if (rows > 1 && need < 2 * cap) cap = (cap + rows - 1) / rows;
+    // Where a row has few descriptors per warp of a full grid, the rows share the chip's places side by side instead:
+    // up to three per warp (12,000 dense kernels against six rows: 148 us, row by row 151; 20,000, 4.1 per warp: 234
+    // against 223), with a work queue up to four (15,000 uneven ones against eight rows: 198 us against 233; 30,000
+    // dense ones against six: 5 % slower). No more CTAs than places: with four above the 608, six rows of 9,000 dense
+    // kernels took 145 us, now 120.
+    if (rows > 1 && need < (p.chunk ? 4 : 3) * cap) cap = std::max<int64_t>(1, cap / rows);
     const int grid = (int)std::min(EMIT ? p.n_kernels : need, cap);
     // By default the first queue counter of the zeroed workspace header.
     if (!queue) queue = queue_word(status, 0);
     EvalParams q = p;
     q.next_row = row + 1 < rows;
+    // A sweep's grabs: about four per warp at least, else the rows end with a few warps that walk long chunks (9,800
+    // dense kernels against six rows, 16 per grab: 288 us, now 130).
+    if (rows > 1 && q.chunk > 1) q.chunk = (int)std::max<int64_t>(1, std::min<int64_t>(q.chunk, p.n_kernels / (4 * kWarps * (int64_t)grid)));
     // emitting: as many descriptors at a time, up to one per warp, as leave each CTA about three turns (the queue
     // evens out spaces of different sizes)
     q.group = (int)std::max<int64_t>(1, std::min<int64_t>(kWarps, p.n_kernels / (3 * cap)));
