@@ -74,6 +74,10 @@ __global__ void features_samples(const __grid_constant__ tune_arch a, const __gr
 // per point that evaluated all 48 features, found its axis values with __fns and wrote its
 // row 4 bytes at a time. 7 CTAs of 4 warps per SM: 72 registers; a full chunk (2^20 points, 8
 // groups a warp) then fills the chip once.
+// Tables are built one kernel after the other, about 3 us each by latency, so where 32 points are of more than
+// kFeatKernels kernels each lane evaluates its point by itself (feat_point). One member, 16,384 kernels, whole call:
+// 1 point each 168 us before the tables, 275 with them alone, 158 now; 4 points 218 / 218 / 190 (eight kernels per
+// 32 points; with the line at 8: 221); 8 points 269 / 239 / 240.
 struct FeatT {
     float t, lane;  // T; 32 W_B / T
     int wb, gw;
@@ -95,6 +99,7 @@ struct FeatC {
     uint16_t b23, b28, b42, pad;
 };
 
+constexpr int kFeatKernels = 4;  // kernels among 32 points up to which their tables are built (see above)
 constexpr int kFeatWarps = 4;
 constexpr int kFeatGroups = 8;  // groups of 32 points a warp walks at most (tables are reused along them)
 
@@ -213,6 +218,30 @@ __device__ __forceinline__ void feat_tables(const tune_arch& a, const Desc& kd, 
     if (lane == 8) s.b43 = bf16_bits((float)s_alloc / 65536.0f);
 }
 
+// The row of point p of descriptor kid by one lane, staged like the others; returns its validity.
+__device__ __forceinline__ bool feat_point(const tune_arch& a, const tune_axes& x, const int4* descs, int64_t kid, int64_t p,
+                                           uint4* row, int sx, int* status)
+{
+    Desc kd;
+    load_desc(descs, kid, kd);
+    const int size = __popc(kd.tm) * __popc(kd.gm) * __popc(kd.um) * __popc(kd.cm);
+    if (desc_bad(kd, x) || p >= size) {
+        atomicOr(status, tune::kStatusInvalid);
+#pragma unroll
+        for (int j = 0; j < kFeatures / 8; ++j) row[j ^ sx] = make_uint4(0, 0, 0, 0);
+        return false;
+    }
+    int tp, gp, up, cp;
+    decode_point(kd, (int)p, tp, gp, up, cp);
+    float f[kFeatures];
+    point_features(a, kd, x.t[tp], x.g[gp], x.u[up], x.c[cp], f);
+#pragma unroll
+    for (int j = 0; j < kFeatures / 8; ++j)
+        row[j ^ sx] = make_uint4(pack2(f[8 * j], f[8 * j + 1]), pack2(f[8 * j + 2], f[8 * j + 3]),
+                                 pack2(f[8 * j + 4], f[8 * j + 5]), pack2(f[8 * j + 6], f[8 * j + 7]));
+    return f[29] > 0.0f;  // B* > 0
+}
+
 // Row i of the chunk = global point p0 + i (p0 = pt_off[k0]) of kernels [k0, k1); a point's
 // kernel is found by a binary search over the offsets (the chunk's few offsets stay in L1).
 // Also writes score[i] = 0 where the point is valid (B* > 0), +inf elsewhere.
@@ -260,6 +289,13 @@ __global__ void __launch_bounds__(32 * kFeatWarps, 7)
         }
         bool valid = false;
         unsigned todo = __ballot_sync(0xffffffffu, on);
+        const int64_t left = __shfl_up_sync(0xffffffffu, lo, 1);
+        const unsigned firsts = __ballot_sync(0xffffffffu, on && (lane == 0 || lo != left));
+        if (__popc(firsts) > kFeatKernels) {
+            if (on) valid = feat_point(a, x, descs, lo, gp - pt_off[lo], row, sx, status);
+            staged = false;
+            todo = 0;
+        }
         while (todo) {
             const int64_t kid = __shfl_sync(0xffffffffu, lo, __ffs(todo) - 1);
             const unsigned mine = __ballot_sync(0xffffffffu, on && lo == kid);
