@@ -545,6 +545,8 @@ extern "C" int surrogate_infer(tune_surrogate* h, const tune_arch* arch, const t
     w += align256(n_kernels * k * 4);
     int64_t* d_off = reinterpret_cast<int64_t*>(w);
 
+    const int64_t sms = tune::device_sm_count();
+    if (sms <= 0) return tune::fail(TUNE_ECUDA, "surrogate_infer: cannot query the SM count");
     TUNE_CUDA_TRY(cudaMemsetAsync(status, 0, tune::kWorkspaceHeader, s), "surrogate_infer: status reset");
     // Analytic top-k of every kernel (the fallback).
     int rc = tune_eval(arch, axes, descs, n_kernels, k, TUNE_SCHED_WARP, a_idx, a_val, nullptr, nullptr, nullptr,
@@ -567,7 +569,7 @@ extern "C" int surrogate_infer(tune_surrogate* h, const tune_arch* arch, const t
         TUNE_CUDA_TRY(cudaGetLastError(), "surrogate_infer: offsets launch");
         if (np > 0) {
             // a warp's walk: long where every SM still gets 16 warps, so that few points stay parallel
-            const int64_t want = np / (32 * 16 * 152);
+            const int64_t want = np / (32 * 16 * sms);
             const int groups = (int)(want < 1 ? 1 : want > kFeatGroups ? kFeatGroups : want);
             const int64_t per_cta = (int64_t)groups * 32 * kFeatWarps;
             features_points<<<(unsigned)((np + per_cta - 1) / per_cta), 32 * kFeatWarps, 0, s>>>(
