@@ -209,8 +209,8 @@ __device__ __forceinline__ unsigned long long merge_lists(const unsigned long lo
     return x;
 }
 
-// Many segments: CTA b owns segments 8 b .. 8 b + 7 of every 8 x grid; its warps take them one after the other
-// from a counter in shared memory, so that a warp with long ones takes fewer. (One queue for the whole
+// Many segments: CTA b owns per = 2^per_log consecutive ones (2, 4 or 8) of every per x grid; its warps take them one
+// after the other from a counter in shared memory, so that a warp with long ones takes fewer. (One queue for the whole
 // grid costs 1.5 ns per segment in atomics on one address: 25 us against 15 for 10,000 segments of 64.) The
 // next segment's bounds are requested before the current one is scanned. Segments longer than kShare, which
 // would keep a warp busy for more than 30 us, are left to the end and shared by the CTA's warps (up to kMaxLong
@@ -218,7 +218,8 @@ __device__ __forceinline__ unsigned long long merge_lists(const unsigned long lo
 constexpr int kShare = 32768, kMaxLong = 64;
 __global__ void __launch_bounds__(kThreads, 4)
     topk_warp_kernel(const float* __restrict__ scores, const int64_t* __restrict__ off, int64_t n_seg, int k,
-                     int32_t* __restrict__ out_i, float* __restrict__ out_s, unsigned char* __restrict__ header)
+                     int per_log, int32_t* __restrict__ out_i, float* __restrict__ out_s,
+                     unsigned char* __restrict__ header)
 {
     static_assert(kThreads == (int)tune::kWorkspaceHeader, "a header byte per thread");
     __shared__ unsigned long long buf[kWarps][64], lists[2][kWarps][kMaxK];
@@ -228,8 +229,10 @@ __global__ void __launch_bounds__(kThreads, 4)
     if (blockIdx.x == 0) header[threadIdx.x] = 0;  // (no separate launch for that)
     if (threadIdx.x == 0) taken = kWarps, n_long = 0;
     __syncthreads();
-    const int64_t stride = (int64_t)gridDim.x * kWarps;
-    auto segment = [&](int i) { return (int64_t)(i / kWarps) * stride + (int64_t)blockIdx.x * kWarps + i % kWarps; };
+    const int per = 1 << per_log;
+    auto segment = [&](int i) {
+        return (((int64_t)(i >> per_log) * gridDim.x + blockIdx.x) << per_log) + (i & (per - 1));
+    };
     int64_t s = segment(warp);
     int64_t b = s < n_seg ? off[s] : 0, e = s < n_seg ? off[s + 1] : 0;
     while (s < n_seg) {
@@ -315,6 +318,8 @@ __global__ void __launch_bounds__(kThreads, 4)
 // many CTAs (2, 4, 8) as there is room for. 64 segments of 16,384 scores (8 CTAs each): 22.8 -> 8.8 us, of
 // 262,144: 143 -> 17.5 us; 600 of 16,384 (1 CTA each) 24.2 -> 11.9 us, where a warp each takes 17; 1,200 of 64
 // (a warp each): 6.8 -> 4.7 us, where a CTA each takes 10.
+// With few more segments than CTAs resident, a CTA owns two or four of them instead of eight, so that all SMs have
+// some (700 of 65,536, k = 5: 39 us on 350 CTAs, 97 on 88; of 16,384: 23 both).
 int launch(const float* scores, const int64_t* off, int64_t n_seg, int k, int32_t* oi, float* os, void* workspace,
            cudaStream_t st)
 {
@@ -326,8 +331,9 @@ int launch(const float* scores, const int64_t* off, int64_t n_seg, int k, int32_
     if (sms <= 0) return tune::fail(TUNE_ECUDA, "tune_topk: cannot query the SM count");
     const int64_t cap = (int64_t)sms * per_sm;
     if (n_seg > cap) {
-        const int64_t need = (n_seg + kWarps - 1) / kWarps;
-        topk_warp_kernel<<<(int)(need < cap ? need : cap), kThreads, 0, st>>>(scores, off, n_seg, k, oi, os,
+        const int per_log = n_seg <= 2 * cap ? 1 : n_seg <= 4 * cap ? 2 : 3;
+        const int64_t need = (n_seg + (1 << per_log) - 1) >> per_log;
+        topk_warp_kernel<<<(int)(need < cap ? need : cap), kThreads, 0, st>>>(scores, off, n_seg, k, per_log, oi, os,
                                                                              static_cast<unsigned char*>(workspace));
         TUNE_CUDA_TRY(cudaGetLastError(), "tune_topk: kernel launch");
         return TUNE_OK;
