@@ -9,6 +9,8 @@
 // list. (Inserting them one by one, with the bound taken from the filling list, cost about 37
 // insertions of some 60 instructions per 3,000-score segment and was what 20,000 ragged segments spent
 // their time on: 92 -> 68 us for 59 M scores with k = 5, 152 -> 62 us with k = 16, the HBM floor being 35.)
+// Short segments have few candidates, which are inserted at their places (k = 1: mostly one), and segments of at most 32
+// scores need no batch: 50,000 of 16 scores 43 -> 25 us with k = 1, 53 -> 25 with k = 5; of 200, k = 1, 45 -> 27.
 //
 // How many warps share a segment (launch()): with more segments than resident CTAs, a warp takes one
 // segment after the other; with fewer segments a whole CTA, or a cluster of up
@@ -29,6 +31,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned long long kNone = ~0ull;  // no entry: behind every key
 constexpr int kVec = 4;                      // 16-byte loads per lane per batch
 constexpr int kBatchF4 = 32 * kVec;          // float4 words per warp batch (2 KB)
+constexpr int kInsert = 8;                   // candidates up to which they are inserted one by one
 constexpr float kFltMax = 3.402823466e+38f;
 
 // Monotone map of non-NaN floats to unsigned integers (-inf smallest, +inf largest).
@@ -96,18 +99,38 @@ struct WarpList {
     {
     }
 
-    // The first 32 buffered candidates into the list. Scores are scanned in increasing index, so once the
-    // list holds k entries a later score has to be below the k-th: the bound steps to the next smaller
-    // float (past -0, which equals +0).
+    // The first 32 buffered candidates into the list.
     __device__ __forceinline__ void flush()
     {
         __syncwarp();
+        if (cnt <= kInsert) {
+            for (int i = 0; i < cnt; ++i) insert(buf[i]);
+            __syncwarp();
+            cnt = 0;
+            bound();
+            return;
+        }
         const unsigned long long x = lane < cnt ? buf[lane] : kNone;
         const unsigned long long more = 32 + lane < cnt ? buf[32 + lane] : kNone;
         __syncwarp();
         if (32 + lane < cnt) buf[lane] = more;
         cnt = max(cnt - 32, 0);
         list = merge32(list, sort32(x, lane), lane);
+        bound();
+    }
+
+    // One entry, the same on every lane, to its place.
+    __device__ __forceinline__ void insert(unsigned long long x)
+    {
+        const int pos = __popc(__ballot_sync(kFull, list < x));
+        const unsigned long long up = __shfl_up_sync(kFull, list, 1);
+        list = lane < pos ? list : lane == pos ? x : up;
+    }
+
+    // Scores are scanned in increasing index, so once the list holds k entries a later score has to be below the
+    // k-th: the bound steps to the next smaller float (past -0, which equals +0).
+    __device__ __forceinline__ void bound()
+    {
         const unsigned tau = (unsigned)(__shfl_sync(kFull, list, k - 1) >> 32);
         if (tau != 0xffffffffu) {
             const unsigned below = tau == 0x80000000u ? 0x7ffffffeu : tau - 1u;
@@ -129,9 +152,15 @@ struct WarpList {
     __device__ __forceinline__ void scan(const Segment& s, int first, int step, bool edges)
     {
         const float nan = __int_as_float(0x7fc00000);
-        if (edges && s.head) {
-            const float v = lane < s.head ? __ldcs(s.p + lane) : nan;
+        // the head, or all of a segment of at most 32 scores, one per lane
+        const int first_n = s.len <= 32 ? s.len : s.head;
+        if (edges && first_n) {
+            const float v = lane < first_n ? __ldcs(s.p + lane) : nan;
             append(v <= thr, v, lane);
+        }
+        if (s.len <= 32) {
+            while (cnt > 0) flush();
+            return;
         }
         const float4* body = reinterpret_cast<const float4*>(s.p + s.head);
         auto load = [&](float4 (&w)[kVec], int f0) {
@@ -161,8 +190,8 @@ struct WarpList {
             for (int j = 1; j < 4 * kVec; ++j) mn = fminf(mn, v[j]);  // fminf skips NaN
             if (fresh) {
                 // k lanes own a score that does not exceed the k-th smallest of the lanes' minima
-                const unsigned key = sort32(mn <= kFltMax ? order_key(mn) : 0xffffffffu, lane);
-                const unsigned kth = __shfl_sync(kFull, key, k - 1);
+                const unsigned key = mn <= kFltMax ? order_key(mn) : 0xffffffffu;
+                const unsigned kth = k == 1 ? __reduce_min_sync(kFull, key) : __shfl_sync(kFull, sort32(key, lane), k - 1);
                 if (kth != 0xffffffffu) thr = fminf(thr, key_value(kth));
                 fresh = false;
             }
