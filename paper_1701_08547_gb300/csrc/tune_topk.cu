@@ -9,6 +9,9 @@
 // list. (Inserting them one by one, with the bound taken from the filling list, cost about 37
 // insertions of some 60 instructions per 3,000-score segment and was what 20,000 ragged segments spent
 // their time on: 92 -> 68 us for 59 M scores with k = 5, 152 -> 62 us with k = 16, the HBM floor being 35.)
+// Where many scores are equal, the bound also drops ties as it goes (10,000 segments of 512 equal scores, k = 16: 64 ->
+// 25 us), and a batch whose scores are mostly below the bound gets one of its own (1,000 falling sequences of 16,384:
+// 348 -> 90 us).
 // Short segments have few candidates, which are inserted at their places (k = 1: mostly one), and segments of at most 32
 // scores need no batch: 50,000 of 16 scores 43 -> 25 us with k = 1, 53 -> 25 with k = 5; of 200, k = 1, 45 -> 27.
 //
@@ -32,6 +35,8 @@ constexpr unsigned long long kNone = ~0ull;  // no entry: behind every key
 constexpr int kVec = 4;                      // 16-byte loads per lane per batch
 constexpr int kBatchF4 = 32 * kVec;          // float4 words per warp batch (2 KB)
 constexpr int kInsert = 8;                   // candidates up to which they are inserted one by one
+constexpr int kMany = 64;                    // candidates of a batch above which they are taken group by group
+constexpr int kLanes = 24;                   // lanes with one above which the batch's own bound is taken again
 constexpr float kFltMax = 3.402823466e+38f;
 
 // Monotone map of non-NaN floats to unsigned integers (-inf smallest, +inf largest).
@@ -73,6 +78,18 @@ __device__ __forceinline__ unsigned long long merge32(unsigned long long a, unsi
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) x = exchange(x, m, (lane & m) == 0);
     return x;
+}
+
+// v[j] by selects (an index would move the array to local memory).
+__device__ __forceinline__ float pick(const float (&v)[4 * kVec], int j)
+{
+    float t[8], u[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t[i] = (j & 1) ? v[2 * i + 1] : v[2 * i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) u[i] = (j & 2) ? t[2 * i + 1] : t[2 * i];
+    const float a = (j & 4) ? u[1] : u[0], b = (j & 4) ? u[3] : u[2];
+    return (j & 8) ? b : a;
 }
 
 // A segment: `head` scores before the first 16-byte boundary, n4 float4 words, the rest from tail0 on.
@@ -188,27 +205,36 @@ struct WarpList {
             float mn = v[0];
 #pragma unroll
             for (int j = 1; j < 4 * kVec; ++j) mn = fminf(mn, v[j]);  // fminf skips NaN
-            if (fresh) {
+            const unsigned who = __ballot_sync(kFull, mn <= thr);
+            if (who == 0u) continue;
+            if (fresh || __popc(who) > kLanes) {
                 // k lanes own a score that does not exceed the k-th smallest of the lanes' minima
                 const unsigned key = mn <= kFltMax ? order_key(mn) : 0xffffffffu;
                 const unsigned kth = k == 1 ? __reduce_min_sync(kFull, key) : __shfl_sync(kFull, sort32(key, lane), k - 1);
                 if (kth != 0xffffffffu) thr = fminf(thr, key_value(kth));
                 fresh = false;
             }
-            if (__ballot_sync(kFull, mn <= thr) == 0u) continue;
             unsigned cm = 0;  // this lane's candidates
 #pragma unroll
             for (int j = 0; j < 4 * kVec; ++j) cm |= v[j] <= thr ? 1u << j : 0u;
-            while (__any_sync(kFull, cm != 0u)) {  // mostly once: a candidate per lane at most
-                const int j = __ffs(cm) - 1;
-                float t[8], u[4];
+            // Mostly a candidate per lane at most, and one turn. Many are mostly ties: those are taken float4 group by
+            // float4 group (128 consecutive scores), and after each the bound, strict for the higher indices of the
+            // groups after it, drops what it excludes.
+            unsigned now = __reduce_add_sync(kFull, __popc(cm)) > kMany ? 0xfu : 0xffffu;
+            for (;;) {
+                const unsigned act = cm & now;
+                if (!__any_sync(kFull, act != 0u)) {
+                    if (now >= 0xf000u) break;
+                    now <<= 4;
+                    if (cm & now) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) t[i] = (j & 1) ? v[2 * i + 1] : v[2 * i];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) u[i] = (j & 2) ? t[2 * i + 1] : t[2 * i];
-                const float a = (j & 4) ? u[1] : u[0], b = (j & 4) ? u[3] : u[2];
-                append(cm != 0u, (j & 8) ? b : a, s.head + 4 * (f0 + lane + 32 * (j >> 2)) + (j & 3));
-                cm &= cm - 1u;
+                        for (int j = 0; j < 4 * kVec; ++j) cm &= v[j] <= thr ? ~0u : ~(1u << j);
+                    }
+                    continue;
+                }
+                const int j = __ffs(act) - 1;
+                append(act != 0u, pick(v, j), s.head + 4 * (f0 + lane + 32 * (j >> 2)) + (j & 3));
+                cm &= ~(act & -act);
                 if (cnt >= 32) flush();
             }
         }
