@@ -86,7 +86,7 @@ def triple_instructions(descs):
 def kernel_source_hash():
     """Hash of the evaluation kernel's sources (tune_eval.cu, the arithmetic and tables it includes)."""
     h = hashlib.sha256()
-    for name in ("tune_eval.cu", "eval_common.cuh", "eval_tables.cuh", "eval_tables.cu"):
+    for name in ("tune_eval.cu", "eval_common.cuh", "eval_tables.cuh", "eval_tables.cu", "f32x2.cuh"):
         with open(os.path.join(ROOT, "paper_1701_08547_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

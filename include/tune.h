@@ -119,7 +119,8 @@ typedef struct tune_kernel_desc {
 #define TUNE_SCHED_THREAD 0x20u /* schedule: one thread per descriptor (not with EMIT) */
 #define TUNE_HOST_DIRECT 0x40u  /* tune_eval_host: evaluate in place in mapped host memory */
 /* Warp schedule knobs (tune_autotune picks them): a work queue handing each warp
- * 2^c consecutive descriptors per grab (c in 0..14; default: a static stride),
+ * 2^c consecutive descriptors per grab (c in 0..14; default: each CTA's warps share the
+ * CTA's own; a sweep's grabs are smaller where a row has few descriptors per warp),
  * and at most m resident CTAs per SM (m in 1..15; default: as many as fit). */
 #define TUNE_SCHED_CHUNK(c) ((((uint32_t)(c)) + 1u) << 8)
 #define TUNE_SCHED_CTAS(m) (((uint32_t)(m)) << 12)
@@ -200,7 +201,7 @@ int tune_eval_noalloc(const tune_arch* arch, const tune_axes* axes, const tune_k
  * tune_autotune — choose tune_eval's schedule for a workload by measurement.
  * (Library tooling; the paper autotunes the kernels it analyses, not itself.)
  * Runs tune_eval on the given descriptors with each candidate schedule — the
- * warp schedule with a static stride or a work queue of 1, 4, 16 or 64
+ * warp schedule with each CTA's own descriptors or a work queue of 1, 4, 16 or 64
  * descriptors per grab at full residency or 2 / 3 CTAs per SM, and the thread
  * schedule — times `reps` runs of each with CUDA events on `stream` (after one
  * untimed run) and keeps the fastest run's time. Returns the winner's schedule

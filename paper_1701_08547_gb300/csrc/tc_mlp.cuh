@@ -52,6 +52,7 @@
 #include <cuda_fp8.h>
 #include <stdint.h>
 
+#include "f32x2.cuh"
 #include "gelu.cuh"
 #include "pdl.cuh"
 #include "tc_gemm.cuh"
@@ -300,27 +301,8 @@ __device__ __forceinline__ void ld16(const float* p, float (&x)[16])
     }
 }
 
-// Packed FP32 pairs (two IEEE single-precision operations, round to nearest, per
-// instruction): the same result in each lane as the scalar fmaf / multiply.
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
-        " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 d;
-    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mul.rn.f32x2 d, a, b;\n"
-        " mov.b64 {%0, %1}, d;\n}\n"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
+using f32x2::fma2;
+using f32x2::mul2;
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
@@ -337,14 +319,6 @@ __device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&w)[8])
         asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "r"(w[0]),
                      "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                      : "memory");
-}
-
-// 256-bit global load of eight floats (address 32-byte aligned; data not written by this kernel).
-__device__ __forceinline__ void ld_global_v8(const float* p, float* x)
-{
-    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
-                 : "l"(p));
 }
 
 // 256-bit global load of eight 32-bit words (address 32-byte aligned; data not written by this kernel),

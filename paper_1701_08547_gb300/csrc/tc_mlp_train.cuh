@@ -9,7 +9,7 @@
 // accumulator at once (which frees it for the next layer) and hand the layer's output over one K chunk at a
 // time, so that the next layer's MMAs start while the later chunks are still being computed. 14 steps of
 // 8,192 rows x 5 members: 2.17 -> 2.05 ms (2.21 with the inference kernel's split of the warps);
-// 1.89 ms with the backward kernels' changes and the L2 policies (policy_evict_first), 1.75 ms with the
+// 1.89 ms with the backward kernels' changes and the L2 policies (policy_evict_first), 1.72 ms with the
 // small launches of a step merged into its large ones.
 #pragma once
 

@@ -26,7 +26,7 @@ extern "C" int tune_autotune(const tune_arch* arch, const tune_axes* axes,
     tune::clear_error();
     if (!best_flags || !best_ms) return tune::fail(TUNE_EINVAL, "best_flags and best_ms must be non-NULL");
     if (reps < 1 || reps > 100) return tune::fail(TUNE_EINVAL, "reps = %d outside [1, 100]", reps);
-    // Candidates: the warp schedule with a static stride or a work queue of
+    // Candidates: the warp schedule with each CTA's own descriptors or a work queue of
     // 1, 4, 16 or 64 descriptors per grab, at full residency or 2 / 3 CTAs per
     // SM; and the thread schedule.
     uint32_t cands[32];

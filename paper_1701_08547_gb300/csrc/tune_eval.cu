@@ -2,11 +2,12 @@
 // terms) over every point of every kernel's tuning space, then per-kernel top-k.
 //
 // Work decomposition (GB300, CUDA cores only; the path is integer/FP32 issue-bound):
-//  * one warp evaluates one kernel descriptor; CTAs of 8 warps stride over the
-//    descriptors (grid = SMs x resident CTAs);
-//  * per CTA, once: tables that depend only on the architecture row and the
-//    axes (W_B, G_W, lane by thread count; hide by W*; waves/slots factor by
-//    (B*, G); floor(w / W_B) for the register limit);
+//  * one warp evaluates one kernel descriptor; the warps of a CTA (eight) take its
+//    descriptors from a counter (grid = SMs x resident CTAs), or a queue hands them
+//    out over the whole grid;
+//  * per CTA, once: a copy of the tables that depend only on the architecture row and
+//    the axes (W_B, G_W, lane by thread count; hide by W*; waves/slots factor by
+//    (B*, G); floor(w / W_B) for the register limit), which the host builds;
 //  * per kernel, lane-parallel: the per-unroll cost sums C_nm(U), C_m(U)
 //    (compensated FP32 sums), register-limited warps, per-carveout G_S, and
 //    the (T, U) block limit min(G_W, G_R);
@@ -42,12 +43,15 @@
 #include <mutex>
 
 #include "eval_tables.cuh"
+#include "f32x2.cuh"
 #include "pdl.cuh"
 #include "tune_internal.h"
 
 namespace {
 
 using namespace tune_dev;
+using f32x2::fma2;
+using f32x2::mul2;
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
@@ -74,7 +78,6 @@ constexpr int kEmitTriples = 240;
 // (200,000 kernels of 128 points each: 511 us by themselves, 824 shared).
 constexpr int kEmitAlone = 2048;
 
-
 struct WarpTables {
     alignas(8) float iparmin[kMaxB + 1];  // by B*: min over the kernel's grid sizes of ipar(B*, G); [0] = NaN
     unsigned short places[kMaxB + 1];  // by B*: the kernel's grid sizes as places in rperm (not for a full set)
@@ -100,35 +103,11 @@ struct WarpTables {
     };
 };
 
-// Sorted insert of (c, i) into a lane's register list (ascending; strict "<"
-// keeps earlier = lower-index entries first among equal costs).
 // (cost, index) keys ordered lexicographically; costs are >= 0, so their bit
 // patterns order like the values.
 __device__ __forceinline__ bool key_less(float c, int i, float c2, int i2)
 {
     return c < c2 || (c == c2 && i < i2);
-}
-
-
-// Packed FP32 pairs (each result rounded to nearest as the scalar operation's).
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
-        " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 d;
-    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mul.rn.f32x2 d, a, b;\n"
-        " mov.b64 {%0, %1}, d;\n}\n"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
 }
 
 template <int N>
@@ -692,7 +671,6 @@ __global__ void __maxnreg__(64)
                     const float mcf = __uint_as_float(mc);
                     if (mc >= 0x7f800000u || mcf > tau0 || mcf > tau_c) break;
                     const unsigned mi = __reduce_min_sync(kFull, h.c == mcf ? (unsigned)h.i : 0xffffffffu);
-                    if (cnt == k && !relaxed && !key_less(mcf, (int)mi, tau_c, tau_i)) break;
                     if (cnt < k && (cnt == 0 || key_less(prev_c, prev_i, mcf, (int)mi))) {
                         if (lane == cnt) {  // in order: append
                             lc = mcf;
@@ -748,12 +726,11 @@ __global__ void __maxnreg__(64)
     if constexpr (EMIT) {
         // A CTA takes `group` descriptors at a time (from the grid's queue), a warp ranks each, and then all its
         // warps write each one's points, an eighth of the thread counts each: the spaces' sizes differ, and a warp
-        // by itself needs 25 us for the points of a full one. (20,000 uneven kernels, 114 M points: 534 us with a
-        // warp per descriptor, lanes on triples and each lane writing its grid sizes nUC points apart; 316 with
-        // the points written in order; 281 shared by the CTA, the HBM floor being 201 (253 now, see below); 6,000 dense ones: 226 -> 181,
-        // 0.96 of the HBM rate.)
-        // Towards the end of the descriptors the groups shrink, to as few as have about 16,384 points (by the mean
-        // of the offsets), so that no CTA is left with eight large spaces: 280 -> 253 us.
+        // by itself needs 25 us for the points of a full one. Towards the end of the descriptors the groups shrink, to
+        // as few as have about 16,384 points (by the mean of the offsets), so that no CTA is left with eight large
+        // spaces. (20,000 uneven kernels, 114 M points: 534 us with a warp per descriptor, lanes on triples and each
+        // lane writing its grid sizes nUC points apart; 316 with the points written in order; 280 shared by the CTA;
+        // 253 with shrinking groups, the HBM floor being 201; 6,000 dense ones: 226 -> 181, 0.96 of the HBM rate.)
         __shared__ long long next;
         __shared__ int next_size;
         const int warp = threadIdx.x >> 5;
