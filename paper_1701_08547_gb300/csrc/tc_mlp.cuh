@@ -19,13 +19,17 @@
 // TMEM lane quarter).
 //
 // What bounds it (2^20 rows x 5 members): an epilogue's 32,768 tanh take the multi-function units 2,048
-// cycles, a layer's MMAs take the tensor cores 2,048; a chain alternates the two, plus the waits
-// between them (100 cycles each alone, 200-350 among busy epilogue warps), about 6,000 cycles per layer
-// of both chains. BF16 2.25 -> 1.84 ms, E4M3 (100,003 rows) 0.192 -> 0.174 ms, against a kernel with the
+// cycles, a layer's MMAs take the tensor cores 2,048; a chain alternates the two, in about 6,000 cycles per
+// layer of both chains. What the rest goes to is not separated: the waits between the two (100 cycles each
+// alone, 200-350 among busy epilogue warps), or the path to shared memory and L1, which carries the MMAs'
+// operand reads in 35 % of the cycles, the epilogues' accesses in 43 % (30 of them parameter loads that hit L1)
+// and the TMA's writes in 24 % (counters, 131,072 rows). BF16 2.25 -> 1.84 ms, E4M3 (100,003 rows) 0.192 ->
+// 0.174 ms, against a kernel with the
 // same roles whose every thread divided 64-bit unit numbers and arrived on the barriers by itself, whose
 // sixteen epilogue warps served the chains in turn with thread = row, and whose single issuing lane
 // could not keep its descriptors in uniform registers (700-900 cycles per chunk of four MMAs, now
-// 480-600). Not kept (best of ten passes, this kernel 1.79 ms): sixteen warps per epilogue with the accumulator loaded at once and handed over
+// 480-600). Not kept (best of ten passes, this kernel 1.79 ms): sixteen warps per epilogue with the accumulator
+// loaded at once and handed over
 // chunk by chunk (1.96 ms here, but the better form for training's few units, tc_mlp_train.cuh); two
 // N = 128 halves (2.26 ms: the A operand is read twice from shared memory); twelve warps of 72
 // registers per chain (1.90 ms); no register split (1.85 ms, spills).
