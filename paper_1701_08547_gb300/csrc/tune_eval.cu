@@ -1069,8 +1069,11 @@ int launch(const EvalParams& p, const tune_kernel_desc* descs, int32_t* ti, floa
     // dense kernels against six rows, 16 per grab: 288 us, now 130).
     if (rows > 1 && q.chunk > 1) q.chunk = (int)std::max<int64_t>(1, std::min<int64_t>(q.chunk, p.n_kernels / (4 * kWarps * (int64_t)grid)));
     // emitting: as many descriptors at a time, up to one per warp, as leave each CTA about three turns (the queue
-    // evens out spaces of different sizes)
-    q.group = (int)std::max<int64_t>(1, std::min<int64_t>(kWarps, p.n_kernels / (3 * cap)));
+    // evens out spaces of different sizes), or one turn where a single array is written: ranking then takes longer than
+    // the stores, and wants all warps (3,000 dense kernels, B* alone: 62 us with three turns, 49 with one, 57 with a
+    // warp per descriptor; all three arrays 101 us with three, 110 with one, 123).
+    const int64_t most = (pb != nullptr) + (pw != nullptr) + (pc != nullptr) > 1 ? p.n_kernels / (3 * cap) : (p.n_kernels + cap - 1) / cap;
+    q.group = (int)std::max<int64_t>(1, std::min<int64_t>(kWarps, most));
     tune::eval_tables(q.a, q.x, q.tab);
     const int4* d = reinterpret_cast<const int4*>(descs);
     if (row > 0)
